@@ -1,4 +1,4 @@
-"""Build libkmq.so in-tree with nvcc for sm_100a (no JIT cache involved)."""
+"""Build libkmq.so and its Python extension module in-tree with nvcc for sm_100a (no JIT cache involved)."""
 from __future__ import annotations
 
 import glob
@@ -6,12 +6,15 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libkmq.so")
+NATIVE_SRC = os.path.join(CSRC, "kmq_python.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_kmq_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
@@ -29,15 +32,15 @@ def sources() -> list[str]:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
+    deps = sources() + [NATIVE_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into libkmq.so; returns its path."""
+    """Compile every .cu under csrc/ into libkmq.so and the extension module beside it; returns the library's path."""
     if not force and not needs_build():
         return LIB_PATH
     os.makedirs(OBJ_DIR, exist_ok=True)
@@ -68,6 +71,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("nvcc failed linking libkmq.so")
     os.replace(LIB_PATH + ".tmp", LIB_PATH)
+
+    # host code only; finds libkmq.so beside itself at run time
+    res = subprocess.run([_nvcc(), "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I",
+                          os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], NATIVE_SRC,
+                          "-L", PKG_DIR, "-l:libkmq.so", "-Xlinker", "-rpath=$ORIGIN", "-o", NATIVE_PATH + ".tmp"],
+                         capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("building the extension module failed")
+    os.replace(NATIVE_PATH + ".tmp", NATIVE_PATH)
     return LIB_PATH
 
 
