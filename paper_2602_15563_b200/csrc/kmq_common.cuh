@@ -30,6 +30,11 @@ __device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
   return v;
 }
 
+__device__ __forceinline__ float4 ldg_stream_f4(const float* p) {
+  const uint4 v = ldg_stream_u4(reinterpret_cast<const uint4*>(p));
+  return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+
 __device__ __forceinline__ void stg_stream_u4(uint4* p, uint4 v) {
   asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");

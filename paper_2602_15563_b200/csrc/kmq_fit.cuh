@@ -1,0 +1,22 @@
+// Fit (and fit fused with assignment and packing): launchers of kmq_fit.cu.
+#pragma once
+#include "kmq_common.cuh"
+
+namespace kmq {
+
+bool fit_supports(int64_t K, int bits);
+
+// One fit per row; centroids may be NULL.
+cudaError_t launch_kmeans_rows(const float* W, int64_t N, int64_t K, int bits, int iters, uint16_t* codebooks,
+                               double* centroids, cudaStream_t s);
+
+// The fit of one codebook on a sample.  Lets the kernel launched next start at once if that asks for it (programmatic
+// dependent launch): that one must not need the codebook.
+cudaError_t launch_fit_sample(const float* values, int64_t count, int bits, int iters, uint16_t* codebook,
+                              cudaStream_t s);
+
+// One fit per row, then the row's weights as packed indices of its stored codebook (bits = 1, 2, 4).
+cudaError_t launch_quantize_rows(const float* W, int64_t N, int64_t K, int bits, int iters, int layout,
+                                 uint16_t* codebooks, uint32_t* packed, cudaStream_t s);
+
+}  // namespace kmq
