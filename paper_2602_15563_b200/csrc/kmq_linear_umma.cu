@@ -25,22 +25,16 @@
 // Every wait on an mbarrier is bounded; a warp whose wait runs out sets bit 0 of the device error word and goes to
 // the end of the kernel (so does, after its own bounded waits, every warp that depended on it); every thread still
 // takes part in the cluster barriers and the final CTA barrier, after which the tensor memory is freed.
-#include <cuda.h>
-
-#include "kmq_common.cuh"
-#include "kmq_linear_variants.cuh"
-#include "kmq_mma_common.cuh"
+#include "kmq_umma_common.cuh"
 
 namespace kmq {
+
+using namespace umma;
 
 __device__ unsigned int g_device_error_flags = 0;   // sticky; read and cleared by kmq_device_error_flags()
 
 namespace {
 
-constexpr int kBM = 128;                                 // output rows per CTA (rows of the MMA)
-constexpr int kDecodeWarps = 16;                         // 4 tensor-memory lane quarters x 4 quarters of a stage's weights
-constexpr int kDecodeThreads = kDecodeWarps * 32;
-constexpr int kThreads = kDecodeThreads + 64;            // + the MMA warp + the TMA producer warp
 // Stages in flight: A operands in tensor memory (the decoders may run this far ahead of the MMAs) and, one per A
 // operand, B buffers in shared memory.  6, or 4 for more than 64 batch rows (128 columns of accumulator, 32 KB per B
 // buffer).
@@ -48,22 +42,6 @@ template <int NB>
 constexpr int ring_depth() {
   return NB > 64 ? 4 : 6;
 }
-constexpr int kWRing = 6;                   // ring of 1 KB steps of packed words per tile (cp.async), kWRing - 1 in flight
-constexpr int kWRowStride = 80;                          // a row's 64 bytes of a step, padded: lanes read consecutive rows
-constexpr int kWStepBytes = kBM * kWRowStride;
-constexpr uint32_t kWaitHintNs = 20000;                  // one try_wait on an mbarrier may park the thread this long
-constexpr uint64_t kWaitLimitNs = 100ull * 1000 * 1000;  // a wait gives up after this much time on the global timer
-
-template <int BITS>
-struct UGeo {
-  static constexpr int kStageK = 128;                            // weights of a row per stage
-  static constexpr int kStagesPerStep = (512 / BITS) / kStageK;  // 1, 2, 4 for b = 4, 2, 1
-  static constexpr int kThreadBytes = kStageK * BITS / 32;       // packed bytes a thread decodes per stage: 16, 8, 4
-  static constexpr int kCols = kStageK / 2;                      // 32-bit columns of the A operand of a stage
-  static constexpr int kKSlices = kStageK / 16;                  // MMAs per stage
-  static constexpr int kTableBytes = BITS == 4 ? 4 * 16 * 128 : 0;   // b = 4: [lane quarter][entry][lane]
-};
-
 template <int BITS, int NB>
 struct USmem {
   static constexpr int kARing = ring_depth<NB>();
@@ -80,188 +58,10 @@ struct USmem {
   static constexpr int kTotal = kTmemSlot + 16 + 1024;   // + room to align the base to 1024 bytes (swizzled B buffers)
 };
 
-// Shared-memory matrix descriptor of a K-major operand in the 128-byte-swizzle layout TMA writes: rows of 128 bytes,
-// 8-row groups 1024 bytes apart (stride byte offset), descriptor version of sm_100, layout type 2 = 128-byte swizzle.
-// The buffer is 1024-byte aligned; 16 weights further along K = 32 bytes further in the start address.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// TMA tile load of the box at (c0, c1) of a 2-D tensor map into shared memory; its bytes complete on `bar`.
-__device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-      : "memory");
-}
-
 // Instruction descriptor of kind::f16: D fp32, A and B bf16, both K-major, M = kBM, N = NB.
 template <int NB>
 __device__ __forceinline__ uint32_t instr_desc() {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
-
-// D (tensor memory) (+)= A (tensor memory) x B (shared memory descriptor)
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// the same with the accumulate flag fixed to true
-__device__ __forceinline__ void umma_bf16_acc(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.eq.u32 p, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_store8(uint32_t taddr, const uint32_t (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(v[0]),
-               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* gmem_src, bool valid) {
-  const int bytes = valid ? 16 : 0;   // 0 source bytes: the 16 destination bytes are zero-filled
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gmem_src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// All threads of all CTAs of the cluster.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The shared::cluster address of CTA 0's copy of this CTA's shared-memory address `saddr`.
-__device__ __forceinline__ uint32_t map_to_rank0(uint32_t saddr) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(saddr));
-  return r;
-}
-// This thread's lane of the accumulator, columns [col0, col0 + NC): all loads are issued before the one wait
-// (zeros when nothing was accumulated).
-template <int NC>
-__device__ __forceinline__ void load_acc(uint32_t (&w)[NC], uint32_t taddr, bool valid) {
-  static_assert(NC % 8 == 0, "whole groups of 8 columns");
-  if (valid) {
-#pragma unroll
-    for (int c = 0; c < NC; c += 8)
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(w[c + 0]), "=r"(w[c + 1]), "=r"(w[c + 2]), "=r"(w[c + 3]), "=r"(w[c + 4]), "=r"(w[c + 5]),
-                     "=r"(w[c + 6]), "=r"(w[c + 7])
-                   : "r"(taddr + c));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-  } else {
-#pragma unroll
-    for (int j = 0; j < NC; ++j) w[j] = 0;
-  }
-}
-
-// Bounded wait for the phase of parity `parity` of an mbarrier.  try_wait parks the thread in hardware for up to the
-// hinted time instead of spinning, so waiting warps do not take issue slots from the ones that decode.  The hint is
-// only a hint (a try may come back early), so the bound is taken on the global timer, not on the number of tries.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  uint64_t t0 = 0;
-  for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity), "r"(kWaitHintNs)
-        : "memory");
-    if (done) return true;
-    uint64_t now;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (t0 == 0) t0 = now;
-    else if (now - t0 > kWaitLimitNs) return false;
-  }
-}
-
-// Decode state of a thread's output row.
-template <int BITS>
-struct RowState;
-template <>
-struct RowState<2> {
-  Dec2 d;
-  __device__ __forceinline__ void init(const uint16_t* cb_row, const unsigned char*, int) { d.init(cb_row); }
-};
-template <>
-struct RowState<1> {
-  uint32_t base, diff;   // (c0, c0) and (c0 ^ c1, c0 ^ c1)
-  __device__ __forceinline__ void init(const uint16_t* cb_row, const unsigned char*, int) {
-    const uint32_t c = __ldg(reinterpret_cast<const uint32_t*>(cb_row));
-    base = prmt(c, c, 0x1010u);
-    diff = base ^ prmt(c, c, 0x3232u);
-  }
-};
-template <>
-struct RowState<4> {
-  const unsigned char* tab;   // this lane's bank of the [entry][lane] table of its lane quarter
-  __device__ __forceinline__ void init(const uint16_t*, const unsigned char* table_quarter, int lane) {
-    tab = table_quarter + lane * 4;
-  }
-};
-
-// One packed word of a row -> bf16 pairs in the order of k, written to consecutive columns of the row's
-// tensor-memory lane starting at `taddr` (8 columns at b = 2, 16 at b = 1).
-template <int BITS>
-__device__ __forceinline__ void decode_word_to_tmem(uint32_t w, const RowState<BITS>& st, uint32_t taddr) {
-  if constexpr (BITS == 2) {
-    uint32_t a[8];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) st.d.pair(w, q, a[2 * q], a[2 * q + 1]);   // weights 4q .. 4q + 3
-    tmem_store8(taddr, a);
-  } else if constexpr (BITS == 1) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t a[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        // shift c puts weights (2c, 2c + 1) on bits 15 and 31; PRMT in sign-replicate mode turns them into
-        // 16-bit masks; the masked XOR picks c0 or c1 bit-exactly
-        const uint32_t sh = w * kPow2[8 * h + i];
-        const uint32_t sel = prmt(sh, sh, 0xBB99u);
-        asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(a[i]) : "r"(sel), "r"(st.diff), "r"(st.base));
-      }
-      tmem_store8(taddr + 8 * h, a);
-    }
-  }
-}
-// b = 4: two words (16 weights) per 8 columns
-__device__ __forceinline__ void decode_words4_to_tmem(uint32_t w0, uint32_t w1, const RowState<4>& st, uint32_t taddr) {
-  uint32_t a[8];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const uint32_t w = j ? w1 : w0;
-    uint32_t e[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {   // nibble i -> byte offset nibble * 128 of the lane's table bank
-      const int sh = 4 * i - 7;
-      const uint32_t u = sh < 0 ? (w << -sh) : (w >> sh);
-      e[i] = *reinterpret_cast<const uint32_t*>(st.tab + (u & 0x780u));
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[4 * j + i] = prmt(e[2 * i], e[2 * i + 1], 0x7610u);
-  }
-  tmem_store8(taddr, a);
 }
 
 template <int BITS, int NB>
@@ -269,7 +69,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
                                                                   const uint16_t* __restrict__ cb,
                                                                   const __grid_constant__ CUtensorMap xmap,
                                                                   uint16_t* __restrict__ y, int64_t N, int64_t K,
-                                                                  int M) {
+                                                                  int64_t M) {
   using G = UGeo<BITS>;
   using SM = USmem<BITS, NB>;
   constexpr int SPS = G::kStagesPerStep;
@@ -288,7 +88,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t block_row0 = (int64_t)blockIdx.x * kBM;
-  const int chunks = (int)(K / (128 / BITS));   // 16-byte chunks per row
+  const int64_t m0 = (int64_t)blockIdx.z * NB;   // first batch row of this CTA's tile
+  const int chunks = (int)((K * BITS + 127) / 128);   // 16-byte chunks per row
   const int steps = (chunks + 3) >> 2;          // the layout pads every row to whole steps of 64 bytes
   // K is split over the gridDim.y CTAs of a cluster (same output rows): rank r takes steps [s_begin, s_end)
   const int ksplit = gridDim.y, rank = blockIdx.y;
@@ -457,8 +258,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
       }
       mbar_expect_tx(full_bar + 8 * buf, SM::kBStageBytes);
       const int k0 = (s_begin * SPS + j) * G::kStageK;
-      tma_load_2d(b_addr + buf * SM::kBStageBytes, &xmap, k0, 0, full_bar + 8 * buf);
-      tma_load_2d(b_addr + buf * SM::kBStageBytes + SM::kBHalfBytes, &xmap, k0 + 64, 0, full_bar + 8 * buf);
+      tma_load_2d(b_addr + buf * SM::kBStageBytes, &xmap, k0, (int)m0, full_bar + 8 * buf);
+      tma_load_2d(b_addr + buf * SM::kBStageBytes + SM::kBHalfBytes, &xmap, k0 + 64, (int)m0, full_bar + 8 * buf);
     }
     if (!ok) atomicOr(&g_device_error_flags, 1u);
   }
@@ -494,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
     for (int j = 0; j < kReadCols; ++j) {
       float v = __uint_as_float(w[j]);
       for (int r = 1; r < ksplit; ++r) v += partial[((r - 1) * NB + col0 + j) * kBM + rho];   // fixed order
-      if (col0 + j < M && n < N) y[(int64_t)(col0 + j) * N + n] = (uint16_t)float_to_bf16_bits(v);
+      if (m0 + col0 + j < M && n < N) y[(m0 + col0 + j) * N + n] = (uint16_t)float_to_bf16_bits(v);
     }
   }
   tc_fence_before_sync();
@@ -512,48 +313,9 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
 
 namespace {
 
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up once through the runtime (no link against the driver library).
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// x as a 2-D tensor [M rows][K] of bf16; boxes of NB rows x 64 columns (128 bytes) land in shared memory with the
-// 128-byte swizzle; rows past M and columns past K read as zero.
-template <int NB>
-bool make_x_map(CUtensorMap* map, const uint16_t* x, int64_t K, int M) {
-  EncodeTiledFn enc = encode_tiled();
-  if (!enc) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
-  const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)NB};
-  const cuuint32_t elem[2] = {1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(x), dims, strides, box, elem,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Dynamic shared memory to launch with: what the kernel uses, but more than half of what an SM offers (the opt-in
-// maximum per CTA is the SM's shared memory minus the 1 KB the system keeps per CTA).
-inline int umma_launch_smem(int kernel_bytes, int max_smem_optin) {
-  const int more_than_half = max_smem_optin / 2 + 1024;
-  return kernel_bytes > more_than_half ? kernel_bytes : more_than_half;
-}
-
 template <int BITS, int NB>
 cudaError_t launch_nb(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N, int64_t K,
-                      int M, cudaStream_t s) {
+                      int64_t M, int ksplit, cudaStream_t s) {
   // Every CTA takes all 512 tensor-memory columns with a blocking tcgen05.alloc and frees them only at its end, after
   // cluster barriers: two such CTAs on one SM (of one cluster or of two) could wait for each other for ever.  The
   // launch therefore asks for more than half of the SM's shared memory whatever the kernel needs, so that a second
@@ -571,13 +333,12 @@ cudaError_t launch_nb(const uint32_t* packed, const uint16_t* cb, const uint16_t
     configured[dev] = true;
   }
   CUtensorMap xmap;
-  if (!make_x_map<NB>(&xmap, x, K, M)) return cudaErrorInvalidValue;
+  if (!make_x_map(&xmap, x, K, M, NB)) return cudaErrorInvalidValue;
   const unsigned blocks = (unsigned)((N + kBM - 1) / kBM);
-  const int ksplit = linear_umma_ksplit(N, K, BITS, NB);
   if ((ksplit - 1) * NB * kBM * 4 > USmem<BITS, NB>::kBRing * USmem<BITS, NB>::kBStageBytes)
     return cudaErrorInvalidValue;   // the partial accumulators of the other CTAs must fit the B buffers
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks, (unsigned)ksplit);
+  cfg.gridDim = dim3(blocks, (unsigned)ksplit, (unsigned)((M + NB - 1) / NB));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -593,26 +354,34 @@ cudaError_t launch_nb(const uint32_t* packed, const uint16_t* cb, const uint16_t
 
 template <int BITS>
 cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
-                        int64_t K, int M, cudaStream_t s) {
-  if (M <= 16) return launch_nb<BITS, 16>(packed, cb, x, y, N, K, M, s);
-  if (M <= 32) return launch_nb<BITS, 32>(packed, cb, x, y, N, K, M, s);
-  if (M <= 48) return launch_nb<BITS, 48>(packed, cb, x, y, N, K, M, s);
-  if (M <= 64) return launch_nb<BITS, 64>(packed, cb, x, y, N, K, M, s);
-  if (M <= 96) return launch_nb<BITS, 96>(packed, cb, x, y, N, K, M, s);
-  return launch_nb<BITS, 128>(packed, cb, x, y, N, K, M, s);
+                        int64_t K, int64_t M, int ksplit, cudaStream_t s) {
+  if (M <= 16) return launch_nb<BITS, 16>(packed, cb, x, y, N, K, M, ksplit, s);
+  if (M <= 32) return launch_nb<BITS, 32>(packed, cb, x, y, N, K, M, ksplit, s);
+  if (M <= 48) return launch_nb<BITS, 48>(packed, cb, x, y, N, K, M, ksplit, s);
+  if (M <= 64) return launch_nb<BITS, 64>(packed, cb, x, y, N, K, M, ksplit, s);
+  if (M <= 96) return launch_nb<BITS, 96>(packed, cb, x, y, N, K, M, ksplit, s);
+  return launch_nb<BITS, 128>(packed, cb, x, y, N, K, M, ksplit, s);
 }
 
 }  // namespace
+}  // namespace kmq
 
-int linear_umma_rows_per_launch() { return 128; }   // one tcgen05.mma costs the same for every N <= 128
+#include "kmq_linear_umma_pair.cuh"
+
+namespace kmq {
+
+// Batch rows per launch (the grid's limits; in earnest one launch).
+constexpr int64_t kSingleMaxRows = 128, kRowsPerLaunch = int64_t(1) << 20;
+int64_t linear_umma_rows_per_launch() { return kRowsPerLaunch; }
 
 // CTAs per 128-row block: K is split over a cluster of 2 or 4 (partial sums meet in CTA 0's shared memory) while the
 // blocks alone would leave at least half (three quarters) of the SMs idle and each part still has a few steps.
 // `batch` = rows of one launch; 4 CTAs only up to 64 rows (three partial accumulators must fit the B buffers).
-int linear_umma_ksplit(int64_t N, int64_t K, int bits, int batch) {
+int linear_umma_ksplit(int64_t N, int64_t K, int bits, int64_t batch) {
   const DeviceInfo* di = device_info();
   if (!di) return 1;
-  const int64_t blocks = (N + kBM - 1) / kBM, steps = (K * bits / 128 + 3) / 4;
+  const int64_t blocks = (N + kBM - 1) / kBM * ((batch + kSingleMaxRows - 1) / kSingleMaxRows);
+  const int64_t steps = (K * bits / 128 + 3) / 4;
   if (blocks * 4 <= di->sm_count && steps >= 32 && batch <= 64) return 4;   // measured: no gain with fewer than 8 steps per CTA
   return (blocks * 2 <= di->sm_count && steps >= 8) ? 2 : 1;
 }
@@ -628,25 +397,49 @@ bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M) {
   // 80 us at 8192 x 28672 for M = 17..32 against 60 us here
   if (!di || M <= (bits == 1 ? 16 : 32) || (K * bits) % 128 != 0) return false;
   if (!encode_tiled()) return false;   // no tensor-map encoder in this driver: stay on the mma.sync kernels
-  const int batch = (int)(M < linear_umma_rows_per_launch() ? M : linear_umma_rows_per_launch());
-  const int64_t ctas = (N + kBM - 1) / kBM * linear_umma_ksplit(N, K, bits, batch);
+  if (M > kSingleMaxRows) return true;
+  const int64_t ctas = (N + kBM - 1) / kBM * linear_umma_ksplit(N, K, bits, M);
   // with fewer CTAs it still wins where the multi-tile kernel is weakest: more than 48 rows, or b = 1 (which that
   // kernel serves 32 rows at a time): 4096 x 4096, 64 CTAs, M = 64: b = 2 18.4 against 20.7 us, b = 1 17.6 against 32.8 us
   const int64_t need = (M > 48 || bits == 1) ? (int64_t)di->sm_count * 3 / 8 : (int64_t)di->sm_count * 5 / 8;
   return ctas >= need;
 }
 
+// Whether more than 128 batch rows go to the CTA pairs.  Clocks, from in-kernel timelines and sweeps: a pair spends 136
+// per 16 weights whatever its batch rows up to 256 (205 at b = 4), 3000 per tile and 8000 per launch besides; a single
+// CTA (up to 128 rows) 115 (225) and 14000, or 24000 where K is split over a cluster, but there are twice as many of
+// them.  The pairs win as soon as their 256 x 256 tiles fill the machine: 16384 x 3072, b = 2, M = 1024: 95 against
+// 164 us; 4096 x 4096, M = 256 (16 tiles): 27 against 20 us.
+static bool pair_pays(int64_t N, int64_t K, int bits, int64_t M) {
+  const DeviceInfo* di = device_info();
+  if (!di || M <= kSingleMaxRows) return false;
+  const int64_t sms = di->sm_count, k16 = K / 16;
+  const int64_t tiles = (N + 2 * kBM - 1) / (2 * kBM) * ((M + kPairMaxRows - 1) / kPairMaxRows);
+  const int64_t rounds = (2 * tiles + sms - 1) / sms;
+  const int64_t pair = 8000 + rounds * (3000 + k16 * (bits == 4 ? 205 : 136));
+  const int64_t ks = linear_umma_ksplit(N, K, bits, M);
+  const int64_t ctas = (N + kBM - 1) / kBM * ((M + kSingleMaxRows - 1) / kSingleMaxRows) * ks;
+  const int64_t single = (ctas + sms - 1) / sms * ((ks > 1 ? 24000 : 14000) + k16 * (bits == 4 ? 225 : 115) / ks);
+  return pair < single;
+}
+
 cudaError_t launch_linear_umma(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                int64_t K, int bits, int64_t M, cudaStream_t s) {
-  const int64_t per = linear_umma_rows_per_launch();
-  for (int64_t m0 = 0; m0 < M; m0 += per) {
-    const int mc = (int)(M - m0 < per ? M - m0 : per);
+  for (int64_t m0 = 0; m0 < M; m0 += kRowsPerLaunch) {
+    const int64_t mc = M - m0 < kRowsPerLaunch ? M - m0 : kRowsPerLaunch;
     const uint16_t* xp = x + m0 * K;
     uint16_t* yp = y + m0 * N;
     cudaError_t e;
-    if (bits == 1) e = launch_bits<1>(packed, cb, xp, yp, N, K, mc, s);
-    else if (bits == 2) e = launch_bits<2>(packed, cb, xp, yp, N, K, mc, s);
-    else e = launch_bits<4>(packed, cb, xp, yp, N, K, mc, s);
+    if (pair_pays(N, K, bits, mc)) {
+      if (bits == 1) e = launch_umma_pair<1>(packed, cb, xp, yp, N, K, mc, s);
+      else if (bits == 2) e = launch_umma_pair<2>(packed, cb, xp, yp, N, K, mc, s);
+      else e = launch_umma_pair<4>(packed, cb, xp, yp, N, K, mc, s);
+    } else {
+      const int ks = linear_umma_ksplit(N, K, bits, mc);
+      if (bits == 1) e = launch_bits<1>(packed, cb, xp, yp, N, K, mc, ks, s);
+      else if (bits == 2) e = launch_bits<2>(packed, cb, xp, yp, N, K, mc, ks, s);
+      else e = launch_bits<4>(packed, cb, xp, yp, N, K, mc, ks, s);
+    }
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

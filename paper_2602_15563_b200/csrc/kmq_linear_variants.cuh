@@ -35,8 +35,8 @@ int linear_multi_min_rows(int bits, int64_t N);   // smallest batch routed to th
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, cudaStream_t s);
 bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M);   // kmq_linear's choice of the tcgen05 kernel
-int linear_umma_rows_per_launch();
-int linear_umma_ksplit(int64_t N, int64_t K, int bits, int batch);   // CTAs (cluster size) per 128-row block
+int64_t linear_umma_rows_per_launch();
+int linear_umma_ksplit(int64_t N, int64_t K, int bits, int64_t batch);   // CTAs (cluster size) per 128-row block
 cudaError_t launch_linear_umma(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                int64_t K, int bits, int64_t M, cudaStream_t s);
 bool linear_lut_supports(int64_t N, int64_t K, int bits, int64_t M);
