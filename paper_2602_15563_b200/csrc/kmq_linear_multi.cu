@@ -10,9 +10,8 @@
 // read from shared memory.  At the end the other K-groups hand their accumulators to the first through shared
 // memory, which adds them, applies the b = 1 codebook and stores bf16.
 //
-// b = 4 uses single-entry per-row tables here (16 entries x 32 lane banks, 4 KB per tile; one LDS per weight and a
-// PRMT per pair): the 64 KB pair tables of the GEMV kernel would not fit for 4 tiles, and the decode is amortised
-// over NT MMAs anyway.
+// The weights are rebuilt in registers at every bit width (Dec1, Dec2, Dec4).  At b = 4 that took the place of per-row
+// tables in shared memory, whose port the B fragments need as well: 8 lookups and up to 8 fragment loads per MMA.
 #include "kmq_common.cuh"
 #include "kmq_linear_variants.cuh"
 #include "kmq_mma_common.cuh"
@@ -20,7 +19,6 @@
 namespace kmq {
 namespace {
 
-constexpr int kTableBytesPerTile = 2 * 16 * 32 * 4;   // b = 4: [half][entry][lane] words
 constexpr int kMaxSmem = 200 * 1024;                  // dynamic shared memory a variant may ask for
 
 template <int BITS>
@@ -39,11 +37,10 @@ template <int BITS, int NT, int TPC, int W = 8>
 struct MSmem {
   using G = MGeo<BITS>;
   static constexpr int kGroups = W / TPC;
-  static constexpr int kTableBytes = BITS == 4 ? TPC * kTableBytesPerTile : 0;
   static constexpr int kBuf = 8 * NT * G::kRowStride;                 // one x buffer: 8 NT batch rows of one step
   static constexpr int kX = kGroups * 2 * kBuf;                       // double buffered, per K-group
   static constexpr int kRed = (kGroups - 1) * TPC * 32 * NT * 4 * 4;  // accumulators of K-groups 1.. (aliases x)
-  static constexpr int kTotal = kTableBytes + (kX > kRed ? kX : kRed);
+  static constexpr int kTotal = kX > kRed ? kX : kRed;
 };
 
 template <int BITS>
@@ -76,8 +73,7 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   constexpr int Q = G::kMmaPerWord;
   constexpr int kGroups = SM::kGroups, kGroupThreads = TPC * 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  unsigned char* const tables = smem_raw;
-  unsigned char* const xbase = smem_raw + SM::kTableBytes;
+  unsigned char* const xbase = smem_raw;
   float* const red = reinterpret_cast<float*>(xbase);                       // reused after the main loop
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -130,15 +126,10 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
     dg.init(cb + min(row0 + g, N - 1) * 4);
     dh.init(cb + min(row0 + g + 8, N - 1) * 4);
   }
+  Dec4 fg, fh;
   if constexpr (BITS == 4) {
-    // word (tile, half, entry e, lane) = C_row[e] in both halves, row = 16 tile + 8 half + lane / 4
-    for (int i = threadIdx.x; i < TPC * 2 * 16 * 32; i += kThreads) {
-      const int ln = i & 31, e = (i >> 5) & 15, half = (i >> 9) & 1, tl = i >> 10;
-      const int64_t r = min(((int64_t)blockIdx.x * TPC + tl) * kTileRows + 8 * half + (ln >> 2), N - 1);
-      const uint32_t c = __ldg(cb + r * 16 + e);
-      reinterpret_cast<uint32_t*>(tables)[i] = c | (c << 16);
-    }
-    __syncthreads();
+    fg.init(cb + min(row0 + g, N - 1) * 16);
+    fh.init(cb + min(row0 + g + 8, N - 1) * 16);
   }
   // Programmatic dependent launch: up to here only the packed indices and the codebooks were read (constants of the
   // layer); the activations may come from the previous kernel on the stream and are read only once it has completed.
@@ -148,8 +139,6 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if constexpr (BITS == 4) asm volatile("griddepcontrol.launch_dependents;");
   if (group < steps) stage(group, 0);
-  const unsigned char* const tab_g = tables + wt * kTableBytesPerTile;   // rows g; rows g + 8 are 2 KB further
-  const uint32_t lane4 = lane * 4;
 
   float acc[NT][4];
 #pragma unroll
@@ -175,6 +164,11 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
       const unsigned char* const xb = xs + g * G::kRowStride + t * G::kChunkStride;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
+        uint32_t dg4[4], dh4[4];
+        if constexpr (BITS == 4) {
+          fg.word(wa[j], dg4);
+          fh.word(wb[j], dh4);
+        }
 #pragma unroll
         for (int q2 = 0; q2 < Q; q2 += 2) {
           uint4 xv[NT];   // 16 bytes of x per batch row = the k-slots of two consecutive MMAs
@@ -189,20 +183,10 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
               dg.pair(wa[j], q, a0, a2);
               dh.pair(wb[j], q, a1, a3);
             } else if constexpr (BITS == 4) {
-              // nibbles 4q .. 4q+3 of the word: weights (4q, 4q+1 | 4q+2, 4q+3); offset = (nibble << 7) | lane * 4
-              uint32_t lo[4], hi[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int sh = 4 * (4 * q + i) - 7;
-                const uint32_t ua = sh < 0 ? (wa[j] << -sh) : (wa[j] >> sh);
-                const uint32_t ub = sh < 0 ? (wb[j] << -sh) : (wb[j] >> sh);
-                lo[i] = *reinterpret_cast<const uint32_t*>(tab_g + and_or(ua, 0x780u, lane4));
-                hi[i] = *reinterpret_cast<const uint32_t*>(tab_g + 2048 + and_or(ub, 0x780u, lane4));
-              }
-              a0 = prmt(lo[0], lo[1], 0x7610u);
-              a2 = prmt(lo[2], lo[3], 0x7610u);
-              a1 = prmt(hi[0], hi[1], 0x7610u);
-              a3 = prmt(hi[2], hi[3], 0x7610u);
+              a0 = dg4[2 * q];
+              a2 = dg4[2 * q + 1];
+              a1 = dh4[2 * q];
+              a3 = dh4[2 * q + 1];
             } else {
               const uint32_t m0 = kPow2[2 * q], m1 = kPow2[2 * q + 1];
               a0 = sg.select(wa[j] * m0);

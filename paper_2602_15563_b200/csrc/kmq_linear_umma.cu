@@ -52,8 +52,7 @@ struct USmem {
   static constexpr int kBStageBytes = 2 * kBHalfBytes;
   static constexpr int kB = 0;
   static constexpr int kWords = kB + kBRing * kBStageBytes;   // ring of packed words: [step][row][80]
-  static constexpr int kTables = kWords + kWRing * kWStepBytes;
-  static constexpr int kBars = kTables + UGeo<BITS>::kTableBytes;   // full[kARing], empty[kARing]
+  static constexpr int kBars = kWords + kWRing * kWStepBytes;   // full[kARing], empty[kARing]
   static constexpr int kTmemSlot = kBars + 2 * kARing * 8;   // then a word that a failed wait sets
   static constexpr int kTotal = kTmemSlot + 16 + 1024;   // + room to align the base to 1024 bytes (swizzled B buffers)
 };
@@ -80,7 +79,6 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
   extern __shared__ __align__(1024) unsigned char smem_unaligned[];
   unsigned char* const smem_raw =
       smem_unaligned + ((1024u - ((uint32_t)__cvta_generic_to_shared(smem_unaligned) & 1023u)) & 1023u);
-  unsigned char* const tables = smem_raw + SM::kTables;
   const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem_raw);
   const uint32_t b_addr = smem_base + SM::kB;
   const uint32_t full_bar = smem_base + SM::kBars, empty_bar = full_bar + 8 * kARing;
@@ -97,7 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
   const int my_steps = s_end - s_begin;
   const int total = my_steps * SPS;             // stages of this CTA
 
-  // ---- set-up: mbarriers, tensor memory, tables ----
+  // ---- set-up: mbarriers, tensor memory ----
   if (threadIdx.x == 0) {
     *reinterpret_cast<volatile uint32_t*>(smem_raw + SM::kTmemSlot + 4) = 0;
 #pragma unroll
@@ -114,15 +112,6 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if constexpr (BITS == 4) {
-    // word [lane quarter q][entry e][lane] = (C_row[e], C_row[e]), row = block_row0 + 32 q + lane
-    for (int i = threadIdx.x; i < 4 * 16 * 32; i += kThreads) {
-      const int ln = i & 31, e = (i >> 5) & 15, q = i >> 9;
-      const int64_t row = min(block_row0 + 32 * q + ln, N - 1);
-      const uint32_t c = __ldg(cb + row * 16 + e);
-      reinterpret_cast<uint32_t*>(tables)[i] = c | (c << 16);
-    }
-  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -138,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
     // row rho % 16 of a tile owns bytes [64 (rho % 16), +64) of each 1 KB step; rows of a tile past N decode zeros
     // and are never stored
     RowState<BITS> st;
-    st.init(cb + min(block_row0 + rho, N - 1) * (1 << BITS), tables + q * 2048, lane);
+    st.d.init(cb + min(block_row0 + rho, N - 1) * (1 << BITS));
     // packed words: whole 1 KB steps of the CTA's 8 tiles, global -> shared, coalesced (thread j copies 16-byte piece
     // j % 64 of tile j / 64 = piece j % 4 of row j / 4), one cp.async group per step, kWRing - 1 steps in flight
     const unsigned char* const w_row = smem_raw + SM::kWords + rho * kWRowStride + kh * G::kThreadBytes;
@@ -190,14 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
         if (!ok) continue;   // up to the next barrier, where all decoders leave
         // this thread's quarter of the stage's weights of its row -> columns kh * kCols / 4 ... of the A operand
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + abuf * G::kCols + kh * (G::kCols / 4);
-        if constexpr (BITS == 4) {
-          decode_words4_to_tmem(wv[0], wv[1], st, taddr);
-          decode_words4_to_tmem(wv[2], wv[3], st, taddr + 8);
-        } else {
-          constexpr int kColsPerWord = 16 / BITS;   // 8 or 16
-#pragma unroll
-          for (int jj = 0; jj < NW; ++jj) decode_word_to_tmem<BITS>(wv[jj], st, taddr + jj * kColsPerWord);
-        }
+        decode_to_tmem<BITS, NW>(wv, st, taddr);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before_sync();
         __syncwarp();
@@ -406,8 +388,8 @@ bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M) {
 }
 
 // Whether more than 128 batch rows go to the CTA pairs.  Clocks, from in-kernel timelines and sweeps: a pair spends 136
-// per 16 weights whatever its batch rows up to 256 (205 at b = 4), 3000 per tile and 8000 per launch besides; a single
-// CTA (up to 128 rows) 115 (225) and 14000, or 24000 where K is split over a cluster, but there are twice as many of
+// per 16 weights whatever its batch rows up to 256 (150 at b = 4), 3000 per tile and 8000 per launch besides; a single
+// CTA (up to 128 rows) 115 (190) and 14000, or 24000 where K is split over a cluster, but there are twice as many of
 // them.  The pairs win as soon as their 256 x 256 tiles fill the machine: 16384 x 3072, b = 2, M = 1024: 95 against
 // 164 us; 4096 x 4096, M = 256 (16 tiles): 27 against 20 us.
 static bool pair_pays(int64_t N, int64_t K, int bits, int64_t M) {
@@ -416,10 +398,10 @@ static bool pair_pays(int64_t N, int64_t K, int bits, int64_t M) {
   const int64_t sms = di->sm_count, k16 = K / 16;
   const int64_t tiles = (N + 2 * kBM - 1) / (2 * kBM) * ((M + kPairMaxRows - 1) / kPairMaxRows);
   const int64_t rounds = (2 * tiles + sms - 1) / sms;
-  const int64_t pair = 8000 + rounds * (3000 + k16 * (bits == 4 ? 205 : 136));
+  const int64_t pair = 8000 + rounds * (3000 + k16 * (bits == 4 ? 150 : 136));
   const int64_t ks = linear_umma_ksplit(N, K, bits, M);
   const int64_t ctas = (N + kBM - 1) / kBM * ((M + kSingleMaxRows - 1) / kSingleMaxRows) * ks;
-  const int64_t single = (ctas + sms - 1) / sms * ((ks > 1 ? 24000 : 14000) + k16 * (bits == 4 ? 225 : 115) / ks);
+  const int64_t single = (ctas + sms - 1) / sms * ((ks > 1 ? 24000 : 14000) + k16 * (bits == 4 ? 190 : 115) / ks);
   return pair < single;
 }
 

@@ -38,8 +38,7 @@ struct PSmem {
   static constexpr int kBStageBytes = 2 * kBHalfBytes;
   static constexpr int kB = 0;
   static constexpr int kWords = kB + kPairRing * kBStageBytes;
-  static constexpr int kTables = kWords + kWRing * kWStepBytes;     // b = 4: of this tile's rows and of the next one's
-  static constexpr int kBars = kTables + 2 * UGeo<BITS>::kTableBytes;
+  static constexpr int kBars = kWords + kWRing * kWStepBytes;
   // full, empty, peer: [kPairRing] each; done, drained
   static constexpr int kTmemSlot = kBars + (3 * kPairRing + 2) * 8;   // then a word that a failed wait sets
   static constexpr int kTotal = kTmemSlot + 16 + 1024;
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
   const int64_t first = blockIdx.x >> 1, stride = gridDim.x >> 1;
   auto row_block = [&](int64_t t) { return 2 * (t % pairs) + rank; };   // this CTA's 128-row block of tile t
 
-  // ---- set-up: mbarriers, tensor memory, tables ----
+  // ---- set-up: mbarriers, tensor memory ----
   if (threadIdx.x == 0) {
     *reinterpret_cast<volatile uint32_t*>(smem_raw + SM::kTmemSlot + 4) = 0;
     auto init = [](uint32_t bar, uint32_t count) {
@@ -132,16 +131,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  // b = 4, by `count` threads: word [lane quarter q][entry e][lane] = (C_row[e], C_row[e]), row = 128 block + 32 q + lane
-  auto build_tables = [&](int64_t block, int buf, int count) {
-    uint32_t* const t = reinterpret_cast<uint32_t*>(smem_raw + SM::kTables + buf * G::kTableBytes);
-    for (int i = threadIdx.x; i < 4 * 16 * 32; i += count) {
-      const int ln = i & 31, e = (i >> 5) & 15, q = i >> 9;
-      const uint32_t c = __ldg(cb + min(block * kBM + 32 * q + ln, N - 1) * 16 + e);
-      t[i] = c | (c << 16);
-    }
-  };
-  if constexpr (BITS == 4) build_tables(row_block(first), 0, kPairThreads);
   tc_fence_before_sync();
   __syncthreads();
   cluster_sync();          // the peer's barriers are set up before anything arrives there
@@ -185,11 +174,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
     for (int d = 0; d < kWRing - 1; ++d) copy_step();
     int slot = 0, abuf = 0;
     uint32_t parity = 1;   // of the wait for an empty stage: the first round finds all of them empty
-    int buf4 = 0;
-    for (int64_t tile = first; tile < tiles && ok; tile += stride, buf4 ^= 1) {
+    for (int64_t tile = first; tile < tiles && ok; tile += stride) {
       RowState<BITS> st;
-      st.init(cb + min(row_block(tile) * kBM + rho, N - 1) * (1 << BITS),
-              smem_raw + SM::kTables + buf4 * G::kTableBytes + q * 2048, lane);
+      st.d.init(cb + min(row_block(tile) * kBM + rho, N - 1) * (1 << BITS));
       for (int s = 0; s < steps; ++s) {
         cp_async_wait<kWRing - 2>();   // this thread's piece of the step has landed
         // every decoder thread's piece has landed, and every one is done with the step before
@@ -199,9 +186,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
           break;
         }
         copy_step();                   // into the slot of the step before
-        if constexpr (BITS == 4) {     // the barriers of the steps to come order this before its use
-          if (s == 0 && tile + stride < tiles) build_tables(row_block(tile + stride), buf4 ^ 1, kDecodeThreads);
-        }
         const unsigned char* const w_step = w_row + slot * kWStepBytes;
         slot = slot + 1 == kWRing ? 0 : slot + 1;
 #pragma unroll
@@ -224,14 +208,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
           }
           if (!ok) continue;   // up to the next barrier, where all decoders leave
           const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + abuf * G::kCols + kh * (G::kCols / 4);
-          if constexpr (BITS == 4) {
-            decode_words4_to_tmem(wv[0], wv[1], st, taddr);
-            decode_words4_to_tmem(wv[2], wv[3], st, taddr + 8);
-          } else {
-            constexpr int kColsPerWord = 16 / BITS;   // 8 or 16
-#pragma unroll
-            for (int jj = 0; jj < NW; ++jj) decode_word_to_tmem<BITS>(wv[jj], st, taddr + jj * kColsPerWord);
-          }
+          decode_to_tmem<BITS, NW>(wv, st, taddr);
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           tc_fence_before_sync();
           __syncwarp();

@@ -65,4 +65,42 @@ struct Dec2 {
   }
 };
 
+// b = 4: the row's 16 centroids as byte tables in registers, l[i] / h[i] = low / high bytes of centroids 4 i .. 4 i + 3.
+// A PRMT looks four indices up in eight entries, so an index below and above 8 is looked up in both halves and the
+// right one chosen by a byte mask made of the indices' top bits (sign-replicating PRMT): 21 integer instructions for
+// the 8 weights of a word and no shared memory.  In kernels whose shared-memory port is taken by MMA operands that
+// beats a table there, one lookup per weight (tcgen05 pairs, 16384 x 3072, M = 1024: 122 us with the table).
+struct Dec4 {
+  uint32_t l[4], h[4];
+  __device__ __forceinline__ void init(const uint16_t* __restrict__ cb_row) {
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(cb_row)), b = __ldg(reinterpret_cast<const uint4*>(cb_row) + 1);
+    l[0] = prmt(a.x, a.y, 0x6420u);
+    h[0] = prmt(a.x, a.y, 0x7531u);
+    l[1] = prmt(a.z, a.w, 0x6420u);
+    h[1] = prmt(a.z, a.w, 0x7531u);
+    l[2] = prmt(b.x, b.y, 0x6420u);
+    h[2] = prmt(b.x, b.y, 0x7531u);
+    l[3] = prmt(b.z, b.w, 0x6420u);
+    h[3] = prmt(b.z, b.w, 0x7531u);
+  }
+  // four indices: selectors in the low half of `sel`, byte i of `m` all ones where index i is 8 or more
+  __device__ __forceinline__ void four(uint32_t sel, uint32_t m, uint32_t& first, uint32_t& second) const {
+    const uint32_t lo = choose(m, prmt(l[0], l[1], sel), prmt(l[2], l[3], sel));
+    const uint32_t hi = choose(m, prmt(h[0], h[1], sel), prmt(h[2], h[3], sel));
+    first = prmt(lo, hi, 0x5140u);
+    second = prmt(lo, hi, 0x7362u);
+  }
+  static __device__ __forceinline__ uint32_t choose(uint32_t m, uint32_t zero, uint32_t one) {
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, 0xB8;" : "=r"(d) : "r"(zero), "r"(m), "r"(one));   // m ? one : zero, bit by bit
+    return d;
+  }
+  // a[i] = weights 2 i, 2 i + 1 of the word
+  __device__ __forceinline__ void word(uint32_t w, uint32_t (&a)[4]) const {
+    const uint32_t sel = w & 0x77777777u, up = w << 4;   // top bits of the even indices to bit 7 of a byte; odd ones are
+    four(sel, prmt(up, w, 0xD9C8u), a[0], a[1]);
+    four(sel >> 16, prmt(up, w, 0xFBEAu), a[2], a[3]);
+  }
+};
+
 }  // namespace kmq

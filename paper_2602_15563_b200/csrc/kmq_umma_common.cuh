@@ -28,7 +28,6 @@ struct UGeo {
   static constexpr int kThreadBytes = kStageK * BITS / 32;       // packed bytes a thread decodes per stage: 16, 8, 4
   static constexpr int kCols = kStageK / 2;                      // 32-bit columns of the A operand of a stage
   static constexpr int kKSlices = kStageK / 16;                  // MMAs per stage
-  static constexpr int kTableBytes = BITS == 4 ? 4 * 16 * 128 : 0;   // b = 4: [lane quarter][entry][lane]
 };
 
 // Shared-memory matrix descriptor of a K-major operand in the 128-byte-swizzle layout TMA writes: rows of 128 bytes,
@@ -163,71 +162,45 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
 template <int BITS>
 struct RowState;
 template <>
-struct RowState<2> {
-  Dec2 d;
-  __device__ __forceinline__ void init(const uint16_t* cb_row, const unsigned char*, int) { d.init(cb_row); }
+struct RowState<1> {
+  Dec1 d;
 };
 template <>
-struct RowState<1> {
-  uint32_t base, diff;   // (c0, c0) and (c0 ^ c1, c0 ^ c1)
-  __device__ __forceinline__ void init(const uint16_t* cb_row, const unsigned char*, int) {
-    const uint32_t c = __ldg(reinterpret_cast<const uint32_t*>(cb_row));
-    base = prmt(c, c, 0x1010u);
-    diff = base ^ prmt(c, c, 0x3232u);
-  }
+struct RowState<2> {
+  Dec2 d;
 };
 template <>
 struct RowState<4> {
-  const unsigned char* tab;   // this lane's bank of the [entry][lane] table of its lane quarter
-  __device__ __forceinline__ void init(const uint16_t*, const unsigned char* table_quarter, int lane) {
-    tab = table_quarter + lane * 4;
-  }
+  Dec4 d;
 };
 
-// One packed word of a row -> bf16 pairs in the order of k, written to consecutive columns of the row's
-// tensor-memory lane starting at `taddr` (8 columns at b = 2, 16 at b = 1).
-template <int BITS>
-__device__ __forceinline__ void decode_word_to_tmem(uint32_t w, const RowState<BITS>& st, uint32_t taddr) {
-  if constexpr (BITS == 2) {
+// The packed words of a row in a stage -> bf16 pairs in the order of k, written to consecutive columns of the row's
+// tensor-memory lane starting at `taddr`.
+template <int BITS, int NW>
+__device__ __forceinline__ void decode_to_tmem(const uint32_t (&w)[NW], const RowState<BITS>& st, uint32_t taddr) {
+  constexpr int kRegs = 16 / BITS * NW;   // 16 per thread and stage
+#pragma unroll
+  for (int c = 0; c < kRegs; c += 8) {
     uint32_t a[8];
+    if constexpr (BITS == 4) {
+      uint32_t x[4], y[4];
+      st.d.word(w[c / 4], x);
+      st.d.word(w[c / 4 + 1], y);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) st.d.pair(w, q, a[2 * q], a[2 * q + 1]);   // weights 4q .. 4q + 3
-    tmem_store8(taddr, a);
-  } else if constexpr (BITS == 1) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t a[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        // shift c puts weights (2c, 2c + 1) on bits 15 and 31; PRMT in sign-replicate mode turns them into
-        // 16-bit masks; the masked XOR picks c0 or c1 bit-exactly
-        const uint32_t sh = w * kPow2[8 * h + i];
-        const uint32_t sel = prmt(sh, sh, 0xBB99u);
-        asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(a[i]) : "r"(sel), "r"(st.diff), "r"(st.base));
+      for (int i = 0; i < 4; ++i) {
+        a[i] = x[i];
+        a[4 + i] = y[i];
       }
-      tmem_store8(taddr + 8 * h, a);
+    } else if constexpr (BITS == 2) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st.d.pair(w[c / 8], q, a[2 * q], a[2 * q + 1]);   // weights 4q .. 4q + 3
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a[i] = st.d.select(w[0] * kPow2[c + i]);   // weights 2 (c + i), 2 (c + i) + 1
     }
+    tmem_store8(taddr + c, a);
   }
 }
-// b = 4: two words (16 weights) per 8 columns
-__device__ __forceinline__ void decode_words4_to_tmem(uint32_t w0, uint32_t w1, const RowState<4>& st, uint32_t taddr) {
-  uint32_t a[8];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const uint32_t w = j ? w1 : w0;
-    uint32_t e[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {   // nibble i -> byte offset nibble * 128 of the lane's table bank
-      const int sh = 4 * i - 7;
-      const uint32_t u = sh < 0 ? (w << -sh) : (w >> sh);
-      e[i] = *reinterpret_cast<const uint32_t*>(st.tab + (u & 0x780u));
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[4 * j + i] = prmt(e[2 * i], e[2 * i + 1], 0x7610u);
-  }
-  tmem_store8(taddr, a);
-}
-
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
