@@ -124,8 +124,7 @@ size_t kmq_workspace_bytes(int64_t N, int64_t K, int bits, int64_t M, int layout
  * of batch rows; 2 for the balanced split with its fix-up kernel), and a short
  * static name of the kernel variant the dispatcher picks: "tiled_*",
  * "split_*", "multi_*", "tcgen05_*" (tuned layout), "table_*" (table layout,
- * bits = 1, 2), "staged_*" (canonical layout),
- * "generic_warp_per_row", or "invalid". */
+ * bits = 1, 2), "staged_*" (canonical layout), or "invalid". */
 int kmq_linear_num_launches(int64_t N, int64_t K, int bits, int64_t M, int layout);
 const char* kmq_linear_variant(int64_t N, int64_t K, int bits, int64_t M, int layout);
 
@@ -286,7 +285,9 @@ kmq_status kmq_dequant_to_bf16(const uint32_t* packed, const uint16_t* codebooks
  *   multiply-accumulate; KMQ_SCALE_DEFERRED ("deferred scaling") accumulates
  *   the 64 unscaled products of a block and scales their sum.  Both are the
  *   same sum up to fp32 rounding and both meet the tolerance stated for
- *   kmq_linear.  x DEVICE bf16 [M,K], y DEVICE bf16 [M,N]; no workspace.
+ *   kmq_linear; on the tensor cores, where a scaled centroid would have to be
+ *   rounded to bf16 first, both are evaluated as the scaled sum.
+ *   x DEVICE bf16 [M,K], y DEVICE bf16 [M,N]; no workspace.
  * kmq_block_dequant_to_bf16 -- W DEVICE bf16 [N,K] = bf16(scale * centroid):
  *   the exact product rounded once, to nearest even (the separate dequantise
  *   step ahead of a standard GEMM, Appendix "Benchmarking", "Model benchmarks").

@@ -71,6 +71,9 @@ __device__ __forceinline__ uint32_t canonical_from_tuned(uint32_t t) {
 
 __host__ __device__ inline int64_t tuned_steps(int64_t wpr) { return (wpr + 15) >> 4; }
 
+// Steps of a row of K weights: the layout pads every row to whole ones.
+__host__ __device__ inline int64_t tuned_row_steps(int64_t K, int bits) { return tuned_steps(K * bits / 32); }
+
 // Index (in 32-bit words) of word j of row n in the tuned layout.
 __host__ __device__ inline int64_t tuned_word_index(int64_t n, int64_t j, int64_t steps) {
   return ((((n >> 4) * steps + (j >> 4)) * kTileRows + (n & 15)) << 4) + (j & 15);

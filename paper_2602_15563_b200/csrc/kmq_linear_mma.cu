@@ -1,22 +1,16 @@
-// kmq_linear on the canonical packed layout, batch rows M <= 8 per pass: one CTA per 16 output rows, the
-// warps of the CTA split K, every warp streams its slices of the packed rows
-// with 128-bit loads (several in flight per lane), rebuilds the bf16 weights
-// in registers directly in the operand layout of mma.sync.m16n8k16 (weights
-// are the 16-row A operand, the batch is the 8-column B operand, fp32
-// accumulators), and the partial sums of the warps are added through shared
+// kmq_linear on the canonical packed layout for b = 1, 2, rows of whole 16-byte chunks and more row tiles than fit the
+// SMs at once (otherwise kmq_rows.cu), up to 4 batch rows: one CTA per 16 output rows, the warps of the CTA
+// split K, every warp streams its slices of the packed rows with 128-bit loads (several in flight per lane), rebuilds
+// the bf16 weights in registers directly in the operand layout of mma.sync.m16n8k16 (weights are the 16-row A operand,
+// the batch is the 8-column B operand, fp32 accumulators), and the partial sums of the warps are added through shared
 // memory before the bf16 store.
 //
-// The integer pipe (64 lane-ops/clk/SM) and the shared-memory port
-// (32 lanes/clk/SM) bound this kernel long before the FMA units do, so each
-// bit width uses the cheapest exact decode that fits them:
-//   b = 2  the row's 4 centroids are 8 bytes = the two source registers of
-//          one byte-permute (PRMT); one PRMT yields two weights.
-//   b = 4  a per-row table of all 256 (centroid, centroid) pairs in shared
-//          memory, one copy per lane bank so lookups never conflict; one
-//          32-bit LDS yields two weights.
-//   b = 1  a shift puts two index bits on bits 15 and 31, a sign-replicating
-//          PRMT spreads them over their half words and one LOP3 selects c0 or
-//          c1: bit copies of the stored centroids.
+// The integer pipe (64 lane-ops/clk/SM) bounds this kernel long before the FMA units do, so each bit width uses the
+// cheapest exact decode for it:
+//   b = 2  the row's 4 centroids are 8 bytes = the two source registers of one byte-permute (PRMT); one PRMT yields two
+//          weights.
+//   b = 1  a shift puts two index bits on bits 15 and 31, a sign-replicating PRMT spreads them over their half words
+//          and one LOP3 selects c0 or c1: bit copies of the stored centroids.
 // The order in which a word's fields reach the k-slots of an MMA is whatever
 // is cheapest to extract; the activations are staged in shared memory in that
 // same order, so the canonical packed layout is consumed as is.
@@ -31,7 +25,6 @@ constexpr int kWarps = 8;          // warps per CTA, all on the same 16 rows, K 
 constexpr int kThreads = kWarps * 32;
 constexpr int kStages = 4;         // 16-byte loads in flight per lane and row
 constexpr int kRows = 16;          // output rows per CTA (one MMA tile)
-constexpr int kPairTableBytes = 32768;  // 256 entries x 32 lane banks x 4 B
 constexpr int kRedBytes = kWarps * 32 * 16;  // per warp: 32 lanes x 4 floats
 
 template <int BITS>
@@ -41,12 +34,11 @@ struct Geo {
   static constexpr int kStepK = 512 / BITS;             // weights of one row consumed per step
   static constexpr int kWordK = 32 / BITS;
   static constexpr int kRowStride = kSlots * 32 + 32;   // bytes of staged activations per batch row (+pad)
-  static constexpr int kTableBytes = BITS == 4 ? 2 * kPairTableBytes : 0;
 };
 
 template <int BITS, int MMAX>
 constexpr int smem_bytes() {
-  return Geo<BITS>::kTableBytes + kWarps * MMAX * Geo<BITS>::kRowStride + kRedBytes;
+  return kWarps * MMAX * Geo<BITS>::kRowStride + kRedBytes;
 }
 
 // ---------------------------------------------------------------------------
@@ -61,12 +53,7 @@ __device__ __forceinline__ void stage_block(const uint16_t* __restrict__ xrow, i
                                             unsigned char* dst) {
   // dst: unit [slot = j*kMmaPerWord][t] of this batch row; consecutive MMAs of the word are 32 bytes apart
   constexpr int Q = Geo<BITS>::kMmaPerWord;
-  if constexpr (BITS == 4) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (valid) v = __ldg(reinterpret_cast<const uint4*>(xrow + k0));
-    *reinterpret_cast<uint2*>(dst) = make_uint2(v.x, v.y);        // weights 0..3 of the word
-    *reinterpret_cast<uint2*>(dst + 32) = make_uint2(v.z, v.w);   // weights 4..7
-  } else if constexpr (BITS == 2) {
+  if constexpr (BITS == 2) {
     uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (valid) {
       const uint4 v0 = __ldg(reinterpret_cast<const uint4*>(xrow + k0));
@@ -120,9 +107,8 @@ __global__ void __launch_bounds__(kThreads) linear_mma_kernel(const uint32_t* __
   using G = Geo<BITS>;
   constexpr int Q = G::kMmaPerWord;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  // [pair tables (b = 4)] [staged activations: kWarps x MMAX rows] [warp partials]
-  unsigned char* const tables = smem_raw;
-  unsigned char* const xs_all = smem_raw + G::kTableBytes;
+  // [staged activations: kWarps x MMAX rows] [warp partials]
+  unsigned char* const xs_all = smem_raw;
   float* const red = reinterpret_cast<float*>(xs_all + kWarps * MMAX * G::kRowStride);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -159,19 +145,10 @@ __global__ void __launch_bounds__(kThreads) linear_mma_kernel(const uint32_t* __
     dg.init(cb + rg * 4);
     dh.init(cb + rh * 4);
   }
-  if constexpr (BITS == 4) {
-    // entry e of row r: (C_r[e & 15], C_r[e >> 4]); the 4 lanes that share a row get one bank each.
-    // Byte address of (half, e, lane) = half * 32 KB + e * 128 + lane * 4, lane = 4 * (r % 8) + t.
-    const int r8 = threadIdx.x & 7, half = (threadIdx.x >> 3) & 1;
-    const int64_t rr = min(row0 + r8 + 8 * half, N - 1);
-    const uint16_t* crow = cb + rr * 16;
-    for (int e = threadIdx.x >> 4; e < 256; e += kThreads / 16) {
-      const uint32_t v = (uint32_t)__ldg(crow + (e & 15)) | ((uint32_t)__ldg(crow + (e >> 4)) << 16);
-      *reinterpret_cast<uint4*>(tables + half * kPairTableBytes + e * 128 + r8 * 16) = make_uint4(v, v, v, v);
-    }
-    __syncthreads();
-  }
-  const uint32_t lane4 = lane * 4;
+  // Programmatic dependent launch: the packed indices and codebooks above are constants of the layer, the activations
+  // may come from the previous kernel on the stream.  The next kernel may start beside this one from here on.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
 
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
 
@@ -205,17 +182,6 @@ __global__ void __launch_bounds__(kThreads) linear_mma_kernel(const uint32_t* __
             if constexpr (BITS == 2) {
               dg.pair(wa[j], q, a0, a2);
               dh.pair(wb[j], q, a1, a3);
-            } else if constexpr (BITS == 4) {
-              // bytes 2q and 2q+1 of the word hold weights (4q, 4q+1) and (4q+2, 4q+3)
-              constexpr uint32_t kMask = 0x7F80u;
-              const uint32_t oa0 = ((q == 0 ? (wa[j] << 7) : (wa[j] >> 9)) & kMask) | lane4;
-              const uint32_t oa1 = ((q == 0 ? (wa[j] >> 1) : (wa[j] >> 17)) & kMask) | lane4;
-              const uint32_t ob0 = ((q == 0 ? (wb[j] << 7) : (wb[j] >> 9)) & kMask) | lane4;
-              const uint32_t ob1 = ((q == 0 ? (wb[j] >> 1) : (wb[j] >> 17)) & kMask) | lane4;
-              a0 = *reinterpret_cast<const uint32_t*>(tables + oa0);
-              a2 = *reinterpret_cast<const uint32_t*>(tables + oa1);
-              a1 = *reinterpret_cast<const uint32_t*>(tables + kPairTableBytes + ob0);
-              a3 = *reinterpret_cast<const uint32_t*>(tables + kPairTableBytes + ob1);
             } else {
               // pair c = 2q: weights (15-2q | 31-2q); pair c = 2q+1: weights (14-2q | 30-2q) on bits 15 and 31
               a0 = sg.select(wa[j] << (2 * q));
@@ -258,9 +224,17 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  const unsigned grid = (unsigned)((N + kRows - 1) / kRows);
-  linear_mma_kernel<BITS, MMAX><<<grid, kThreads, smem, s>>>(packed, cb, x, y, N, K, M);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((N + kRows - 1) / kRows));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, linear_mma_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M);
 }
 
 template <int BITS>
@@ -268,31 +242,24 @@ cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16
                         int64_t K, int M, cudaStream_t s) {
   if (M == 1) return launch_one<BITS, 1>(packed, cb, x, y, N, K, M, s);
   if (M == 2) return launch_one<BITS, 2>(packed, cb, x, y, N, K, M, s);
-  if (M <= 4) return launch_one<BITS, 4>(packed, cb, x, y, N, K, M, s);
-  return launch_one<BITS, 8>(packed, cb, x, y, N, K, M, s);
+  return launch_one<BITS, 4>(packed, cb, x, y, N, K, M, s);
 }
 
 }  // namespace
 
-bool linear_mma_supports(int64_t N, int64_t K, int bits, int64_t M) {
-  (void)M;
-  return (K * bits) % 128 == 0 && K <= (int64_t(1) << 30) && (N + kRows - 1) / kRows <= 0x7FFFFFFF;
+// Against kmq_rows.cu (whose lanes load 2 or 4 bytes at b = 1, 2 where these load 16, but stage nothing): faster with
+// more tiles than resident CTAs and up to 4 batch rows (8192 x 8192: M = 1, b = 1 11.5 / 17.2 us, b = 2 13.7 / 17.4 us;
+// M = 4, b = 2 17.3 / 17.9 us; M = 8 23.9 / 18 us), slower below (4096 x 4096, b = 2: 5.0 / 4.8 us).
+bool linear_mma_selected(int64_t N, int64_t K, int bits, int64_t M) {
+  const DeviceInfo* di = device_info();
+  return bits != 4 && M <= 4 && (K * bits) % 128 == 0 && di && (N + kRows - 1) / kRows > 2 * (int64_t)di->sm_count;
 }
 
-// Batches larger than 8 are processed 8 rows at a time (one launch each).
+// At most 4 batch rows.
 cudaError_t launch_linear_mma(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                               int64_t K, int bits, int64_t M, cudaStream_t s) {
-  for (int64_t m0 = 0; m0 < M; m0 += 8) {
-    const int mc = (int)(M - m0 < 8 ? M - m0 : 8);
-    const uint16_t* xp = x + m0 * K;
-    uint16_t* yp = y + m0 * N;
-    cudaError_t e;
-    if (bits == 1) e = launch_bits<1>(packed, cb, xp, yp, N, K, mc, s);
-    else if (bits == 2) e = launch_bits<2>(packed, cb, xp, yp, N, K, mc, s);
-    else e = launch_bits<4>(packed, cb, xp, yp, N, K, mc, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  if (bits == 1) return launch_bits<1>(packed, cb, x, y, N, K, (int)M, s);
+  return launch_bits<2>(packed, cb, x, y, N, K, (int)M, s);
 }
 
 }  // namespace kmq

@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   const int64_t tile_id = (int64_t)blockIdx.x * TPC + wt;
   const bool has_tile = tile_id < tiles;               // warp-uniform; such a warp still stages x and joins barriers
   const int64_t row0 = tile_id * kTileRows;
-  const int chunks = (int)(K / (4 * G::kWordK));
-  const int steps = (chunks + 3) >> 2;
+  const int steps = (int)tuned_row_steps(K, BITS);
   const uint4* __restrict__ tile =
       reinterpret_cast<const uint4*>(packed) + (has_tile ? tile_id : 0) * (int64_t)steps * 64 + lane;
   unsigned char* const xgroup = xbase + group * 2 * SM::kBuf;
@@ -273,7 +272,7 @@ cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16
   const bool fits_one_wave = (tiles + 3) / 4 <= (di ? di->sm_count : 148);   // CTAs of 4 tiles <= SMs
   // few tiles and a long K: 2 tiles x 8 K-groups (16 warps) while each K-group still gets 4 steps or more
   // (4096 x 11008, b = 2, M = 16: 13.4 -> 12.3 us; 4096 x 4096: b = 4 11.5 -> 9.8 us, b = 2 (16 steps) 6.4 -> 6.9 us)
-  const bool few16 = few && (tiles + 1) / 2 <= (di ? di->sm_count : 148) && (K * BITS / 128 + 3) / 4 >= 32;
+  const bool few16 = few && (tiles + 1) / 2 <= (di ? di->sm_count : 148) && tuned_row_steps(K, BITS) >= 32;
   if (M <= 8) {
     // same shape of CTA for up to 8 batch rows (8192 x 28672, b = 1, M = 4: 35.0 -> 23.5 us; 8192 x 8192, b = 2,
     // M = 8: 12.7 -> 11.7 us)

@@ -83,8 +83,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int64_t row0 = tile_id * kRows;
-  const int chunks = (int)(K / (4 * G::kWordK));   // 16-byte chunks per row
-  const int steps = (chunks + 3) >> 2;             // the layout pads every row to whole steps
+  const int steps = (int)tuned_row_steps(K, BITS);
   // step s of this tile: 64 16-byte units, unit h * 32 + lane = row (g + 8h), chunk t
   const uint4* __restrict__ tile = reinterpret_cast<const uint4*>(packed) + tile_id * steps * 64 + lane;
   __syncthreads();   // a previous segment's readers of the tables and of `red` are done
@@ -275,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_tiled_kernel(c
                                                                     const uint16_t* __restrict__ x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, int early) {
-  const int steps = (int)((K / (4 * TGeo<BITS>::kWordK) + 3) >> 2);
+  const int steps = (int)tuned_row_steps(K, BITS);
   const int64_t row0 = (int64_t)blockIdx.x * kRows;
   float v;
   tile_segment<BITS, MMAX>(packed, cb, x, N, K, M, blockIdx.x, 0, steps, true, early != 0, v);
@@ -301,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_split_kernel(c
                                                                     const uint16_t* __restrict__ x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, float* __restrict__ scratch) {
-  const int64_t steps = (K / (4 * TGeo<BITS>::kWordK) + 3) >> 2;
+  const int64_t steps = tuned_row_steps(K, BITS);
   const int64_t units = ((N + kRows - 1) / kRows) * steps;
   const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
   bool first = true;   // the first segment waits for the previous kernel on the stream before it reads x
@@ -327,7 +326,7 @@ __global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const flo
                                                                        const uint16_t* __restrict__ cb,
                                                                        uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                        int M, int ctas) {
-  const int64_t steps = (K / (4 * TGeo<BITS>::kWordK) + 3) >> 2;
+  const int64_t steps = tuned_row_steps(K, BITS);
   const int64_t units = ((N + kRows - 1) / kRows) * steps;
   const int64_t cut = units * (blockIdx.x + 1) / ctas;
   if (cut % steps == 0) return;   // the cut is a tile boundary: nothing was left partial
@@ -382,7 +381,7 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const DeviceInfo* di = device_info();
-  const int64_t steps = (K / (4 * TGeo<BITS>::kWordK) + 3) >> 2;
+  const int64_t steps = tuned_row_steps(K, BITS);
   const int early = di && early_trigger(BITS, (N + kRows - 1) / kRows, steps, di->sm_count) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, linear_tiled_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M, early);
 }
@@ -509,7 +508,7 @@ int linear_split_ctas(int64_t N, int64_t K, int bits, int64_t M) {
   if (per_sm <= 0) return 0;
   const int64_t slots = (int64_t)di->sm_count * per_sm;
   const int64_t tiles = (N + kRows - 1) / kRows;
-  const int64_t steps = (K * bits / 128 + 3) / 4;
+  const int64_t steps = tuned_row_steps(K, bits);
   return (tiles > slots && steps >= kSplitMinSteps) ? (int)slots : 0;
 }
 

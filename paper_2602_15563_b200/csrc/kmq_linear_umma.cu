@@ -87,8 +87,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t block_row0 = (int64_t)blockIdx.x * kBM;
   const int64_t m0 = (int64_t)blockIdx.z * NB;   // first batch row of this CTA's tile
-  const int chunks = (int)((K * BITS + 127) / 128);   // 16-byte chunks per row
-  const int steps = (chunks + 3) >> 2;          // the layout pads every row to whole steps of 64 bytes
+  const int steps = (int)tuned_row_steps(K, BITS);
   // K is split over the gridDim.y CTAs of a cluster (same output rows): rank r takes steps [s_begin, s_end)
   const int ksplit = gridDim.y, rank = blockIdx.y;
   const int s_begin = (int)((int64_t)steps * rank / ksplit), s_end = (int)((int64_t)steps * (rank + 1) / ksplit);
@@ -363,7 +362,7 @@ int linear_umma_ksplit(int64_t N, int64_t K, int bits, int64_t batch) {
   const DeviceInfo* di = device_info();
   if (!di) return 1;
   const int64_t blocks = (N + kBM - 1) / kBM * ((batch + kSingleMaxRows - 1) / kSingleMaxRows);
-  const int64_t steps = (K * bits / 128 + 3) / 4;
+  const int64_t steps = tuned_row_steps(K, bits);
   if (blocks * 4 <= di->sm_count && steps >= 32 && batch <= 64) return 4;   // measured: no gain with fewer than 8 steps per CTA
   return (blocks * 2 <= di->sm_count && steps >= 8) ? 2 : 1;
 }
@@ -377,7 +376,7 @@ bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M) {
   const DeviceInfo* di = device_info();
   // b = 1: the multi-tile kernel has no 16-warp form beyond 16 rows (its x buffers are twice as large) and takes
   // 80 us at 8192 x 28672 for M = 17..32 against 60 us here
-  if (!di || M <= (bits == 1 ? 16 : 32) || (K * bits) % 128 != 0) return false;
+  if (!di || M <= (bits == 1 ? 16 : 32)) return false;
   if (!encode_tiled()) return false;   // no tensor-map encoder in this driver: stay on the mma.sync kernels
   if (M > kSingleMaxRows) return true;
   const int64_t ctas = (N + kBM - 1) / kBM * linear_umma_ksplit(N, K, bits, M);

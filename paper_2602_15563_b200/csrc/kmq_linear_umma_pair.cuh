@@ -102,8 +102,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x & 1;                       // the pair = two neighbouring 128-row blocks
-  const int chunks = (int)((K * BITS + 127) / 128);      // 16-byte chunks per row
-  const int steps = (chunks + 3) >> 2;                   // the layout pads every row to whole steps of 64 bytes
+  const int steps = (int)tuned_row_steps(K, BITS);
   const int total = steps * SPS;                         // stages per tile
   // tile t: row pair t % pairs, batch tile t / pairs; this pair of CTAs takes tiles first, first + stride, ...
   const int64_t pairs = (N + 2 * kBM - 1) / (2 * kBM), tiles = pairs * ((M + NB - 1) / NB);

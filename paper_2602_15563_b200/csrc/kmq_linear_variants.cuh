@@ -5,8 +5,8 @@
 namespace kmq {
 
 enum LinearVariant : int {
-  kVariantGeneric = 0,   // any legal shape and layout, CUDA-core FMAs, one warp per output row
-  kVariantMma = 1,       // canonical layout, K*bits % 128 == 0: tensor-core GEMV, activations staged per warp
+  kVariantRows = 1,      // canonical layout: tensor-core GEMV, operands straight from global memory
+  kVariantMma = 0,       // canonical layout, b = 1, 2, many row tiles: tensor-core GEMV, activations staged per warp
   kVariantTiled = 2,     // tuned (tile-major) layout: tensor-core GEMV with coalesced 1 KB steps, small batches (M <= 8)
   kVariantMulti = 3,     // tuned layout, M >= linear_multi_min_rows(): 32 or 64 rows per CTA share the staged
                          // activations, one decode feeds up to 8 MMAs
@@ -17,10 +17,7 @@ enum LinearVariant : int {
   kVariantUnsupported = 7,
 };
 
-cudaError_t launch_linear_generic(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
-                                  int64_t K, int bits, int64_t M, int layout, cudaStream_t s);
-
-bool linear_mma_supports(int64_t N, int64_t K, int bits, int64_t M);
+bool linear_mma_selected(int64_t N, int64_t K, int bits, int64_t M);
 cudaError_t launch_linear_mma(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                               int64_t K, int bits, int64_t M, cudaStream_t s);
 cudaError_t launch_linear_tiled(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,

@@ -1,0 +1,318 @@
+// The layer on row-major packed weights, on the tensor cores: kmq_linear on the canonical layout (any K) and
+// kmq_block_linear (shared codebook, scale per block of 64 inputs).
+//
+// A CTA owns 16 output rows; its warps take the row's groups of 64 inputs in turn.  Lane (g, t) of a warp owns inputs
+// 16 t .. 16 t + 15 of a group for rows g and g + 8 and for batch row g: 16 b bits of packed indices per row (2 to 16
+// bytes, neighbouring lanes neighbouring bytes) and 32 bytes of x, loaded straight into registers.
+// The inputs of an MMA's 16 k-slots are chosen to fit: MMA s (of 4 per group) takes inputs 4 s .. 4 s + 3 of every
+// lane's 16, so that both its A and its B fragment are register pairs the lane already holds, in the order in which the
+// indices are packed; nothing is staged or permuted.  (m16n8k16: weights are the 16-row A operand, up to 8 batch rows
+// per B operand, NT B operands per A.)
+// An A register is two weights: one lookup of the index pair in a shared-memory table with a copy per lane bank
+// (b = 8: two single lookups).  In the block format the table is the same for all rows, and the four MMAs of a group
+// make the unscaled sum of a block, which is scaled once in fp32: an exact product of scale and centroid does not fit a
+// bf16 operand, so both scale orders of the interface are evaluated this way; they differ by fp32 rounding only.
+// What bounds it: the lookups and their addresses, 8 integer instructions and 4 shared loads per 256 weights, next to
+// NT MMAs; on short rows the latency of a few dependent loads.  4096 x 4096, block format, b = 4, M = 8: 30 us on the
+// FMA units (2 passes over the weights, 5 instructions per weight).
+#include "kmq_rows.cuh"
+
+#include "kmq_mma_common.cuh"
+
+namespace kmq {
+namespace {
+
+constexpr int kGroup = 64;   // inputs of a group (= a block of the block format)
+
+template <int BITS, bool BLOCK>
+struct RGeo {
+  static constexpr int kPairBits = BITS == 8 ? 8 : 2 * BITS;              // index bits of a lookup
+  static constexpr int kEntries = 1 << kPairBits;
+  static constexpr int kHalf = BLOCK ? 0 : kEntries * 128;                // table of rows g + 8 (block format: the same)
+  static constexpr int kTableBytes = kEntries * 128 * (BLOCK ? 1 : 2);    // entry e, lane l at e * 128 + 4 l
+  static constexpr int kWords = BITS >= 2 ? BITS / 2 : 1;                 // 32-bit words of 16 indices (b = 1: half of one)
+};
+
+// Groups that a warp loads together and then works on.  A rolling ring (load the group three ahead, use the oldest) was
+// slower: the loads a warp waits for share their scoreboards with the newest ones.  8192 x 8192, block format, b = 4,
+// M = 1: ring of 3 27.0 us, 1 / 2 / 4 groups at a time 20.6 / 19.5 / 20.5 us; 4096 x 4096: 8.9 and 8.1 / 7.8 / 7.3 us.
+template <int NT>
+struct Batch {
+  static constexpr int kGroups = NT == 1 ? 4 : 1;
+};
+
+template <int BITS, bool BLOCK>
+struct Indices {
+  uint32_t wa[RGeo<BITS, BLOCK>::kWords], wb[RGeo<BITS, BLOCK>::kWords];
+  uint32_t sa, sb;   // block format: bf16 scales of rows g, g + 8
+};
+
+// The lane's 16 indices of one row at `p`; of a canonical row's last group only what lies inside the row.
+template <int BITS, bool BLOCK>
+__device__ __forceinline__ void load_indices(const uint8_t* p, int left, uint32_t (&w)[RGeo<BITS, BLOCK>::kWords]) {
+#pragma unroll
+  for (int i = 0; i < RGeo<BITS, BLOCK>::kWords; ++i) w[i] = 0;
+  if (left <= 0) return;
+  if constexpr (BITS == 1) {
+    w[0] = __ldg(reinterpret_cast<const uint16_t*>(p));
+  } else if constexpr (BITS == 2) {
+    w[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+  } else if constexpr (BITS == 4 && BLOCK) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+  } else if constexpr (BITS == 4) {      // rows are whole words, no more
+    w[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+    if (left > 8) w[1] = __ldg(reinterpret_cast<const uint32_t*>(p) + 1);
+  } else {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
+  }
+}
+
+// Weights 2 j, 2 j + 1 of the lane's 16 as one register.
+template <int BITS, bool BLOCK>
+__device__ __forceinline__ uint32_t weight_pair(const uint32_t (&w)[RGeo<BITS, BLOCK>::kWords], int j,
+                                                const unsigned char* table, uint32_t lane4) {
+  using G = RGeo<BITS, BLOCK>;
+  auto lookup = [&](int bit) {           // the field at `bit` of the 16 indices, as byte offset field * 128 + 4 lane
+    const uint32_t word = w[bit >> 5];
+    const int at = (bit & 31) - 7;
+    const uint32_t u = at < 0 ? word << -at : word >> at;
+    return *reinterpret_cast<const uint32_t*>(table + and_or(u, (uint32_t)(G::kEntries - 1) << 7, lane4));
+  };
+  if constexpr (BITS == 8) return prmt(lookup(16 * j), lookup(16 * j + 8), 0x5410u);
+  else return lookup(G::kPairBits * j);
+}
+
+template <int BITS, bool BLOCK, int NT, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_kernel(const uint8_t* __restrict__ wq,
+                                                                 const uint16_t* __restrict__ scales,
+                                                                 const uint16_t* __restrict__ cb,
+                                                                 const uint16_t* __restrict__ x,
+                                                                 uint16_t* __restrict__ y, int64_t N, int64_t K, int M) {
+  using G = RGeo<BITS, BLOCK>;
+  constexpr int AHEAD = Batch<NT>::kGroups;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* const table = smem_raw;
+  float* const red = reinterpret_cast<float*>(smem_raw);   // after the main loop: [warp][NT][32 lanes][4]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int64_t row0 = (int64_t)blockIdx.x * kTileRows;
+  const int64_t ra = min(row0 + g, N - 1), rb = min(row0 + g + 8, N - 1);   // rows past the end are not stored
+  const int64_t row_bytes = K * BITS / 8;
+  const int groups = (int)((K + kGroup - 1) / kGroup);
+  const uint8_t* const pa = wq + ra * row_bytes + t * 2 * BITS;
+  const uint8_t* const pb = wq + rb * row_bytes + t * 2 * BITS;
+  const uint16_t* const px = x + 16 * t;
+
+  auto left_of = [&](int gi) {   // inputs of the lane's 16 inside the row
+    return BLOCK ? 16 : (int)min((int64_t)16, K - ((int64_t)gi * kGroup + 16 * t));
+  };
+  auto load_weights = [&](int gi, Indices<BITS, BLOCK>& q) {
+    const int left = left_of(gi);
+    load_indices<BITS, BLOCK>(pa + (int64_t)gi * 8 * BITS, left, q.wa);
+    load_indices<BITS, BLOCK>(pb + (int64_t)gi * 8 * BITS, left, q.wb);
+    if constexpr (BLOCK) {
+      q.sa = __ldg(scales + ra * groups + gi);
+      q.sb = __ldg(scales + rb * groups + gi);
+    }
+  };
+  auto load_x = [&](int gi, uint32_t (&q)[NT][8]) {
+    const int left = left_of(gi);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      const int m = 8 * nt + g;
+      const uint4* const src = reinterpret_cast<const uint4*>(px + (int64_t)m * K + (int64_t)gi * kGroup);
+      uint4 v = make_uint4(0, 0, 0, 0), u = make_uint4(0, 0, 0, 0);
+      if (m < M && left > 0) v = __ldg(src);
+      if (m < M && left > 8) u = __ldg(src + 1);
+      q[nt][0] = v.x; q[nt][1] = v.y; q[nt][2] = v.z; q[nt][3] = v.w;
+      q[nt][4] = u.x; q[nt][5] = u.y; q[nt][6] = u.z; q[nt][7] = u.w;
+    }
+  };
+  // Programmatic dependent launch.  Packed indices and codebooks of kmq_linear are constants of the layer: the first
+  // batch of them and the tables do not wait for the previous kernel on the stream; the activations do, and so does
+  // everything in the block format, whose interface says nothing of the kind.
+  if constexpr (BLOCK) asm volatile("griddepcontrol.wait;" ::: "memory");
+  Indices<BITS, BLOCK> first[AHEAD];
+  if constexpr (!BLOCK) {
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d)
+      if (warp + d * WARPS < groups) load_weights(warp + d * WARPS, first[d]);
+  }
+
+  // ---- tables ----
+  if constexpr (BLOCK) {
+    for (int i = threadIdx.x; i < G::kEntries * 8; i += WARPS * 32) {   // four lanes' copies of an entry at a time
+      const int e = i >> 3;
+      const uint32_t lo = __ldg(cb + (BITS == 8 ? e : e & ((1 << BITS) - 1)));
+      const uint32_t v = BITS == 8 ? lo : lo | ((uint32_t)__ldg(cb + (e >> BITS)) << 16);
+      reinterpret_cast<uint4*>(table)[i] = make_uint4(v, v, v, v);
+    }
+  } else {
+    constexpr int Q = 1 << BITS;
+    for (int i = threadIdx.x; i < 16 * Q; i += WARPS * 32) {            // row r, low index: the entries of all high ones
+      const int r = i & 15, low = i >> 4;
+      const uint16_t* const c = cb + min(row0 + r, N - 1) * Q;
+      const uint32_t lo = __ldg(c + low);
+      unsigned char* const dst = table + (r >> 3) * G::kHalf + low * 128 + (r & 7) * 16;
+#pragma unroll
+      for (int hi = 0; hi < Q; ++hi) {
+        const uint32_t v = lo | ((uint32_t)__ldg(c + hi) << 16);
+        *reinterpret_cast<uint4*>(dst + hi * Q * 128) = make_uint4(v, v, v, v);
+      }
+    }
+  }
+  __syncthreads();
+  if constexpr (!BLOCK) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The next kernel on the stream may start beside this one (4096 x 4096, b = 2: 5.5 us with the release at the end, 4.8).
+  asm volatile("griddepcontrol.launch_dependents;");
+
+  const uint32_t lane4 = lane * 4;
+  float acc[NT][4];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+  // groups g0, g0 + WARPS, ... of a batch
+  auto multiply = [&](int g0, const Indices<BITS, BLOCK> (&w)[AHEAD]) {
+    uint32_t xs[AHEAD][NT][8];
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d)
+      if (g0 + d * WARPS < groups) load_x(g0 + d * WARPS, xs[d]);
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d) {
+      if (g0 + d * WARPS < groups) {   // uniform over the warp
+        const Indices<BITS, BLOCK>& q = w[d];
+        float part[NT][4];
+        if constexpr (BLOCK) {
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) part[nt][0] = part[nt][1] = part[nt][2] = part[nt][3] = 0.f;
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const uint32_t a0 = weight_pair<BITS, BLOCK>(q.wa, 2 * s, table, lane4);
+          const uint32_t a2 = weight_pair<BITS, BLOCK>(q.wa, 2 * s + 1, table, lane4);
+          const uint32_t a1 = weight_pair<BITS, BLOCK>(q.wb, 2 * s, table + G::kHalf, lane4);
+          const uint32_t a3 = weight_pair<BITS, BLOCK>(q.wb, 2 * s + 1, table + G::kHalf, lane4);
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+            mma_bf16_16816(BLOCK ? part[nt] : acc[nt], a0, a1, a2, a3, xs[d][nt][2 * s], xs[d][nt][2 * s + 1]);
+        }
+        if constexpr (BLOCK) {
+          const float sa = bf16_bits_to_float(q.sa), sb = bf16_bits_to_float(q.sb);
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            acc[nt][0] = fmaf(sa, part[nt][0], acc[nt][0]);
+            acc[nt][1] = fmaf(sa, part[nt][1], acc[nt][1]);
+            acc[nt][2] = fmaf(sb, part[nt][2], acc[nt][2]);
+            acc[nt][3] = fmaf(sb, part[nt][3], acc[nt][3]);
+          }
+        }
+      }
+    }
+  };
+  int g0 = warp;
+  if constexpr (!BLOCK) {
+    multiply(g0, first);
+    g0 += AHEAD * WARPS;
+  }
+  for (; g0 < groups; g0 += AHEAD * WARPS) {
+    Indices<BITS, BLOCK> batch[AHEAD];   // of this round only: nothing of it lives on to the next
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d)
+      if (g0 + d * WARPS < groups) load_weights(g0 + d * WARPS, batch[d]);
+    multiply(g0, batch);
+  }
+  // ---- the warps' sums, in warp order ----
+  __syncthreads();   // the tables give way
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+    *reinterpret_cast<float4*>(red + ((warp * NT + nt) * 32 + lane) * 4) =
+        make_float4(acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
+  __syncthreads();
+  for (int i = threadIdx.x; i < NT * 128; i += WARPS * 32) {
+    const int r = i & 15, m = i >> 4;   // consecutive threads -> consecutive output rows
+    const int src = ((m >> 3) * 32 + (r & 7) * 4 + ((m & 7) >> 1)) * 4 + (r >> 3) * 2 + (m & 1);
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) v += red[w * NT * 128 + src];
+    if (m < M && row0 + r < N) y[(int64_t)m * N + row0 + r] = (uint16_t)float_to_bf16_bits(v);
+  }
+}
+
+template <int BITS, bool BLOCK, int NT, int WARPS>
+cudaError_t launch_one(const uint8_t* wq, const uint16_t* scales, const uint16_t* cb, const uint16_t* x, uint16_t* y,
+                       int64_t N, int64_t K, int M, cudaStream_t s) {
+  constexpr int table = RGeo<BITS, BLOCK>::kTableBytes, red = WARPS * NT * 512;
+  constexpr int smem = table > red ? table : red;
+  static bool configured[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !configured[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(linear_rows_kernel<BITS, BLOCK, NT, WARPS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    configured[dev] = true;
+  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((N + kTileRows - 1) / kTileRows));
+  cfg.blockDim = dim3(WARPS * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, linear_rows_kernel<BITS, BLOCK, NT, WARPS>, wq, scales, cb, x, y, N, K, M);
+}
+
+template <int BITS, bool BLOCK>
+cudaError_t launch_passes(const uint8_t* wq, const uint16_t* scales, const uint16_t* cb, const uint16_t* x, uint16_t* y,
+                          int64_t N, int64_t K, int64_t M, cudaStream_t s) {
+  const DeviceInfo* di = device_info();
+  if (!di) return cudaErrorInvalidDevice;
+  const bool few = (N + kTileRows - 1) / kTileRows <= di->sm_count;   // at most a CTA per SM: 16 warps share its K
+  const int per = BLOCK ? 32 : linear_rows_per_launch();
+  for (int64_t m0 = 0; m0 < M; m0 += per) {
+    const int mc = (int)(M - m0 < per ? M - m0 : per);
+    const uint16_t* xp = x + m0 * K;
+    uint16_t* yp = y + m0 * N;
+    cudaError_t e;
+    if (!BLOCK || mc <= 8)
+      e = few ? launch_one<BITS, BLOCK, 1, 16>(wq, scales, cb, xp, yp, N, K, mc, s)
+              : launch_one<BITS, BLOCK, 1, 8>(wq, scales, cb, xp, yp, N, K, mc, s);
+    else if (mc <= 16)
+      e = few ? launch_one<BITS, true, 2, 16>(wq, scales, cb, xp, yp, N, K, mc, s)
+              : launch_one<BITS, true, 2, 8>(wq, scales, cb, xp, yp, N, K, mc, s);
+    else
+      e = few ? launch_one<BITS, true, 4, 16>(wq, scales, cb, xp, yp, N, K, mc, s)
+              : launch_one<BITS, true, 4, 8>(wq, scales, cb, xp, yp, N, K, mc, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+int linear_rows_per_launch() { return 8; }   // the canonical layout is not meant for batches: tuned layout
+
+cudaError_t launch_linear_rows(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
+                               int64_t K, int bits, int64_t M, cudaStream_t s) {
+  const uint8_t* wq = reinterpret_cast<const uint8_t*>(packed);
+  if (bits == 1) return launch_passes<1, false>(wq, nullptr, cb, x, y, N, K, M, s);
+  if (bits == 2) return launch_passes<2, false>(wq, nullptr, cb, x, y, N, K, M, s);
+  return launch_passes<4, false>(wq, nullptr, cb, x, y, N, K, M, s);
+}
+
+cudaError_t launch_block_rows(const uint8_t* wq, const uint16_t* scales, const uint16_t* codebook, const uint16_t* x,
+                              uint16_t* y, int64_t N, int64_t K, int bits, int64_t M, cudaStream_t s) {
+  if (bits == 1) return launch_passes<1, true>(wq, scales, codebook, x, y, N, K, M, s);
+  if (bits == 2) return launch_passes<2, true>(wq, scales, codebook, x, y, N, K, M, s);
+  if (bits == 4) return launch_passes<4, true>(wq, scales, codebook, x, y, N, K, M, s);
+  return launch_passes<8, true>(wq, scales, codebook, x, y, N, K, M, s);
+}
+
+}  // namespace kmq
