@@ -1,4 +1,5 @@
 // extern "C" boundary of libkmq: argument validation and dispatch.
+#include <atomic>
 #include <mutex>
 
 #include "kmq_common.cuh"
@@ -10,18 +11,19 @@ namespace kmq {
 const DeviceInfo* device_info() {
   constexpr int kMaxDevices = 64;
   static DeviceInfo cache[kMaxDevices];
-  static bool valid[kMaxDevices] = {};
+  static std::atomic<bool> valid[kMaxDevices];
   static std::mutex mu;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  if (valid[dev].load(std::memory_order_acquire)) return &cache[dev];
   std::lock_guard<std::mutex> lock(mu);
-  if (!valid[dev]) {
+  if (!valid[dev].load(std::memory_order_relaxed)) {
     int sms = 0, smem = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     if (cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return nullptr;
     cache[dev].sm_count = sms;
     cache[dev].max_smem_optin = smem;
-    valid[dev] = true;
+    valid[dev].store(true, std::memory_order_release);
   }
   return &cache[dev];
 }
@@ -138,6 +140,32 @@ kmq_status kmq_unpack(const uint32_t* packed, int64_t N, int64_t K, int bits, in
 
 namespace {
 
+// The plan of a call depends on its shape and the device only, and a program comes back with the same few shapes: each
+// thread remembers the last plan for some of them (working one out takes a third of a microsecond, a tenth of a call).
+const LinearPlan& cached_plan(const DeviceInfo* di, int64_t N, int64_t K, int bits, int64_t M, int layout) {
+  struct Entry {
+    const DeviceInfo* di;
+    int64_t N, K, M;
+    int bits, layout;
+    LinearPlan plan;
+  };
+  constexpr int kEntries = 64;
+  static thread_local Entry cache[kEntries] = {};
+  const uint64_t h = ((uint64_t)N * 0x9E3779B97F4A7C15u) ^ ((uint64_t)K * 0xC2B2AE3D27D4EB4Fu) ^
+                     ((uint64_t)(M * 16 + bits * 4 + layout) * 0x165667B19E3779F9u);
+  Entry& e = cache[h >> 58];
+  if (e.di != di || e.N != N || e.K != K || e.M != M || e.bits != bits || e.layout != layout) {
+    e.plan = plan_linear(N, K, bits, M, layout);
+    e.di = di;
+    e.N = N;
+    e.K = K;
+    e.M = M;
+    e.bits = bits;
+    e.layout = layout;
+  }
+  return e.plan;
+}
+
 // Every check of kmq_linear that needs no GPU work; on success `plan` is the kernel variant to launch.
 kmq_status check_linear_args(const uint32_t* packed, const uint16_t* codebooks, const uint16_t* x, const uint16_t* y,
                              int64_t N, int64_t K, int bits, int64_t M, int layout, const void* workspace,
@@ -146,8 +174,9 @@ kmq_status check_linear_args(const uint32_t* packed, const uint16_t* codebooks, 
   if (kmq_status s = check_shape(N, K, bits, M)) return s;
   if (!known_layout(layout)) return KMQ_ERR_LAYOUT;
   if (!aligned16(packed) || !aligned16(codebooks) || !aligned16(x) || !aligned16(y)) return KMQ_ERR_ALIGN;
-  if (!device_info()) return KMQ_ERR_CUDA;
-  *plan = plan_linear(N, K, bits, M, layout);
+  const DeviceInfo* const di = device_info();
+  if (!di) return KMQ_ERR_CUDA;
+  *plan = cached_plan(di, N, K, bits, M, layout);
   if (plan->workspace > 0) {
     if (!workspace || workspace_bytes < plan->workspace) return KMQ_ERR_WORKSPACE;
     if (!aligned16(workspace)) return KMQ_ERR_ALIGN;
@@ -179,10 +208,17 @@ kmq_status kmq_linear_host(const uint32_t* packed, const uint16_t* codebooks, co
                                        workspace_bytes, &plan))
     return s;
   cudaStream_t st = (cudaStream_t)stream;
-  if (cudaMemcpyAsync(x_dev, x_host, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess) return KMQ_ERR_CUDA;
+  const size_t x_bytes = (size_t)M * K * 2, y_bytes = (size_t)M * N * 2;
+  void* const x_mapped = host_copy_address(x_host, x_bytes);
+  void* const y_mapped = host_copy_address(y_host, y_bytes);
+  if ((x_mapped ? launch_host_copy(x_dev, x_mapped, x_bytes, st)
+                : cudaMemcpyAsync(x_dev, x_host, x_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+    return KMQ_ERR_CUDA;
   if (launch_linear(plan, packed, codebooks, x_dev, y_dev, N, K, bits, M, layout, workspace, st) != cudaSuccess)
     return KMQ_ERR_CUDA;
-  if (cudaMemcpyAsync(y_host, y_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess) return KMQ_ERR_CUDA;
+  if ((y_mapped ? launch_host_copy(y_mapped, y_dev, y_bytes, st)
+                : cudaMemcpyAsync(y_host, y_dev, y_bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+    return KMQ_ERR_CUDA;
   return cudaStreamSynchronize(st) == cudaSuccess ? KMQ_OK : KMQ_ERR_CUDA;
 }
 

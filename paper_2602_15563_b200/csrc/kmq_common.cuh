@@ -97,6 +97,10 @@ cudaError_t launch_unpack(const uint32_t* packed, int64_t N, int64_t K, int bits
 cudaError_t launch_dequant(const uint32_t* packed, const uint16_t* cb, uint16_t* W, int64_t N, int64_t K, int bits,
                            int layout, cudaStream_t s);
 
+// kmq_host_copy.cu: copies by a kernel between pinned host memory and the device
+void* host_copy_address(const void* host, size_t bytes);   // nullptr: use cudaMemcpyAsync
+cudaError_t launch_host_copy(void* dst, const void* src, size_t bytes, cudaStream_t s);
+
 struct LinearPlan {
   int variant;        // index into the variant table
   int launches;       // kernels launched per call
