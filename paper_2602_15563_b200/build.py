@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import shutil
 import subprocess
@@ -29,6 +30,11 @@ def _nvcc() -> str:
 
 def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def _torch_include() -> str:
+    """torch's header folder (the extension module uses its DLPack header), found without importing torch."""
+    return os.path.join(os.path.dirname(importlib.util.find_spec("torch").origin), "include")
 
 
 def needs_build() -> bool:
@@ -74,7 +80,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     # host code only; finds libkmq.so beside itself at run time
     res = subprocess.run([_nvcc(), "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I",
-                          os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], NATIVE_SRC,
+                          os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", _torch_include(), NATIVE_SRC,
                           "-L", PKG_DIR, "-l:libkmq.so", "-Xlinker", "-rpath=$ORIGIN", "-o", NATIVE_PATH + ".tmp"],
                          capture_output=True, text=True)
     if res.returncode != 0:

@@ -55,6 +55,12 @@ extern "C" {
 
 int kmq_version(void) { return 100; }
 
+// For the Python extension module: the device that the library's calls on this thread go to.
+int kmq_internal_current_device(void) {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
 const char* kmq_status_string(int status) {
   switch (status) {
     case KMQ_OK: return "ok";
