@@ -10,8 +10,12 @@
 // read from shared memory.  At the end the other K-groups hand their accumulators to the first through shared
 // memory, which adds them, applies the b = 1 codebook and stores bf16.
 //
-// The weights are rebuilt in registers at every bit width (Dec1, Dec2, Dec4).  At b = 4 that took the place of per-row
-// tables in shared memory, whose port the B fragments need as well: 8 lookups and up to 8 fragment loads per MMA.
+// The weights are rebuilt in registers (Dec1, Dec2, Dec4).  At b = 4 that costs 2.6 integer instructions a weight, and up
+// to 16 batch rows the integer pipe bounded the kernel (72 % busy, the shared-memory port 28 %): there the upper 8 rows of
+// a tile come from tables of all 256 (centroid, centroid) pairs in shared memory, half an instruction and half a load a
+// weight, and the lower 8 from registers, so that both pipes carry a part (8192 x 28672, us per call before / after:
+// M = 4 57.3 / 47.1, M = 16 65.0 / 54.2; 4096 x 4096, M = 16: 8.0 / 7.1).  With more batch rows the port is taken by the
+// activations' fragments.
 #include "kmq_common.cuh"
 #include "kmq_linear_variants.cuh"
 #include "kmq_mma_common.cuh"
@@ -20,6 +24,9 @@ namespace kmq {
 namespace {
 
 constexpr int kMaxSmem = 200 * 1024;                  // dynamic shared memory a variant may ask for
+// Pair table of 8 rows: entry e, lane l (the 4 lanes of a row get a bank each) at e * 256 + l * 4; two tables interleave.
+constexpr int kEntryStride = 256;
+constexpr int kHalfTableBytes = 256 * kEntryStride / 2;
 
 template <int BITS>
 struct MGeo {
@@ -40,7 +47,9 @@ struct MSmem {
   static constexpr int kBuf = 8 * NT * G::kRowStride;                 // one x buffer: 8 NT batch rows of one step
   static constexpr int kX = kGroups * 2 * kBuf;                       // double buffered, per K-group
   static constexpr int kRed = (kGroups - 1) * TPC * 32 * NT * 4 * 4;  // accumulators of K-groups 1.. (aliases x)
-  static constexpr int kTotal = kX > kRed ? kX : kRed;
+  static constexpr bool kTab = BITS == 4 && NT <= 2;                   // pair tables of the tiles' upper 8 rows
+  static constexpr int kTables = kTab ? TPC * kHalfTableBytes : 0;
+  static constexpr int kTotal = kTables + (kX > kRed ? kX : kRed);
 };
 
 template <int BITS>
@@ -73,7 +82,7 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   constexpr int Q = G::kMmaPerWord;
   constexpr int kGroups = SM::kGroups, kGroupThreads = TPC * 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  unsigned char* const xbase = smem_raw;
+  unsigned char* const xbase = smem_raw + SM::kTables;
   float* const red = reinterpret_cast<float*>(xbase);                       // reused after the main loop
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -127,9 +136,29 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   }
   Dec4 fg, fh;
   if constexpr (BITS == 4) {
-    fg.init(cb + min(row0 + g, N - 1) * 16);
+    if constexpr (!SM::kTab) fg.init(cb + min(row0 + g, N - 1) * 16);
     fh.init(cb + min(row0 + g + 8, N - 1) * 16);
   }
+  if constexpr (SM::kTab) {
+    // a thread takes a row and a low index: one fetch of the row's centroids, the 16 entries low + 16 high
+    for (int it = threadIdx.x; it < TPC * 128; it += kThreads) {
+      const int r8 = it & 7, low = (it >> 3) & 15, i = it >> 7;
+      const int64_t row = min(((int64_t)blockIdx.x * TPC + i) * kTileRows + r8, N - 1);
+      const uint16_t* const crow = cb + row * 16;
+      const uint4 ca = __ldg(reinterpret_cast<const uint4*>(crow)), cc = __ldg(reinterpret_cast<const uint4*>(crow) + 1);
+      const uint32_t lo = __ldg(crow + low);
+      const uint32_t c2[8] = {ca.x, ca.y, ca.z, ca.w, cc.x, cc.y, cc.z, cc.w};
+      unsigned char* const dst = smem_raw + (i >> 1) * (2 * kHalfTableBytes) + (i & 1) * 128 + low * kEntryStride + r8 * 16;
+#pragma unroll
+      for (int hi = 0; hi < 16; ++hi) {
+        const uint32_t v = prmt(lo, c2[hi >> 1], (hi & 1) ? 0x7610u : 0x5410u);
+        *reinterpret_cast<uint4*>(dst + hi * 16 * kEntryStride) = make_uint4(v, v, v, v);
+      }
+    }
+    __syncthreads();
+  }
+  // this lane's bank of the tile's table; byte 1 is the entry's place
+  const uint32_t bank = (wt >> 1) * (2 * kHalfTableBytes) + (wt & 1) * 128 + lane * 4;
   // Programmatic dependent launch: up to here only the packed indices and the codebooks were read (constants of the
   // layer); the activations may come from the previous kernel on the stream and are read only once it has completed.
   // At b = 4, where the set-up of a CTA is long (its tables), the next kernel is released at once so that its CTAs
@@ -165,7 +194,7 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
       for (int j = 0; j < 4; ++j) {
         uint32_t dg4[4], dh4[4];
         if constexpr (BITS == 4) {
-          fg.word(wa[j], dg4);
+          if constexpr (!SM::kTab) fg.word(wa[j], dg4);
           fh.word(wb[j], dh4);
         }
 #pragma unroll
@@ -182,8 +211,16 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
               dg.pair(wa[j], q, a0, a2);
               dh.pair(wb[j], q, a1, a3);
             } else if constexpr (BITS == 4) {
-              a0 = dg4[2 * q];
-              a2 = dg4[2 * q + 1];
+              if constexpr (SM::kTab) {
+                // index byte k of the word in byte 1 of `bank`
+                const uint32_t o0 = prmt(wa[j], bank, 0x7604u | ((2 * q) << 4));
+                const uint32_t o1 = prmt(wa[j], bank, 0x7604u | ((2 * q + 1) << 4));
+                a0 = *reinterpret_cast<const uint32_t*>(smem_raw + o0);
+                a2 = *reinterpret_cast<const uint32_t*>(smem_raw + o1);
+              } else {
+                a0 = dg4[2 * q];
+                a2 = dg4[2 * q + 1];
+              }
               a1 = dh4[2 * q];
               a3 = dh4[2 * q + 1];
             } else {
