@@ -117,7 +117,8 @@ int64_t kmq_packed_bit_index(int64_t n, int64_t k, int plane, int64_t N, int64_t
 int kmq_preferred_layout(int64_t N, int64_t K, int bits, int64_t M);
 
 /* Bytes of scratch kmq_linear needs for this shape on the current device
- * (fp32 partial sums of a split along K); may be 0. */
+ * (fp32 partial sums of a split along K); may be 0.  Batches that could run
+ * without (the "multi_balanced_*" kernels) do so when a call brings less. */
 size_t kmq_workspace_bytes(int64_t N, int64_t K, int bits, int64_t M, int layout);
 
 /* Number of kernels one kmq_linear call launches for this shape (one per pass

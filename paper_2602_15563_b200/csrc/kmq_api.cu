@@ -183,6 +183,8 @@ kmq_status check_linear_args(const uint32_t* packed, const uint16_t* codebooks, 
   const DeviceInfo* const di = device_info();
   if (!di) return KMQ_ERR_CUDA;
   *plan = cached_plan(di, N, K, bits, M, layout);
+  // a call that comes with less scratch than the fastest plan uses may still be served by one that uses less
+  if (plan->workspace > (workspace ? workspace_bytes : 0)) *plan = plan_linear(N, K, bits, M, layout, 0);
   if (plan->workspace > 0) {
     if (!workspace || workspace_bytes < plan->workspace) return KMQ_ERR_WORKSPACE;
     if (!aligned16(workspace)) return KMQ_ERR_ALIGN;

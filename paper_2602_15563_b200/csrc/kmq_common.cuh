@@ -108,7 +108,8 @@ struct LinearPlan {
   int split_k;        // K slices (1 = none)
   const char* name;
 };
-LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout);
+// `scratch_limit`: plans that only gain by scratch, not need it, are left out beyond this.
+LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout, size_t scratch_limit = ~size_t(0));
 cudaError_t launch_linear(const LinearPlan& plan, const uint32_t* packed, const uint16_t* cb, const uint16_t* x,
                           uint16_t* y, int64_t N, int64_t K, int bits, int64_t M, int layout, void* workspace,
                           cudaStream_t s);

@@ -5,7 +5,7 @@
 
 namespace kmq {
 
-LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout) {
+LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout, size_t scratch_limit) {
   LinearPlan p;
   p.workspace = 0;
   p.split_k = 1;
@@ -43,6 +43,13 @@ LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout) {
     p.variant = kVariantMulti;
     p.launches = (int)((M + per - 1) / per);
     p.name = bits == 4 ? "multi_prmt_b4" : bits == 2 ? "multi_prmt_b2" : "multi_select_b1";
+    const MultiSplit sp = linear_multi_split(N, K, bits, M);
+    if (sp.ctas && scratch_limit >= sp.scratch) {
+      p.launches = 2;
+      p.split_k = sp.ctas;
+      p.workspace = sp.scratch;
+      p.name = bits == 4 ? "multi_balanced_b4" : bits == 2 ? "multi_balanced_b2" : "multi_balanced_b1";
+    }
     return p;
   }
   if (const int ctas = linear_split_ctas(N, K, bits, M)) {
@@ -73,7 +80,7 @@ cudaError_t launch_linear(const LinearPlan& plan, const uint32_t* packed, const 
     case kVariantUmma:
       return launch_linear_umma(packed, cb, x, y, N, K, bits, M, s);
     case kVariantMulti:
-      return launch_linear_multi(packed, cb, x, y, N, K, bits, M, s);
+      return launch_linear_multi(packed, cb, x, y, N, K, bits, M, plan.workspace ? workspace : nullptr, s);
     case kVariantMma:
       return launch_linear_mma(packed, cb, x, y, N, K, bits, M, s);
     case kVariantRows:

@@ -16,6 +16,8 @@
 // weight, and the lower 8 from registers, so that both pipes carry a part (8192 x 28672, us per call before / after:
 // M = 4 57.3 / 47.1, M = 16 65.0 / 54.2; 4096 x 4096, M = 16: 8.0 / 7.1).  With more batch rows the port is taken by the
 // activations' fragments.
+#include <atomic>
+
 #include "kmq_common.cuh"
 #include "kmq_linear_variants.cuh"
 #include "kmq_mma_common.cuh"
@@ -70,12 +72,30 @@ __device__ __forceinline__ void group_barrier(int group, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(threads) : "memory");
 }
 
-template <int BITS, int NT, int TPC, int W = 8>
-__global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 1) linear_multi_kernel(const uint32_t* __restrict__ packed,
-                                                                    const uint16_t* __restrict__ cb,
-                                                                    const uint16_t* __restrict__ x,
-                                                                    uint16_t* __restrict__ y, int64_t N, int64_t K,
-                                                                    int M) {
+// This lane's four sums of 8 batch rows from `m0` on -> y (rows row0 + g, + 8; batch rows m0 + 2 t, + 1).
+__device__ __forceinline__ void store_sums(const float (&v)[4], uint16_t* __restrict__ y, int64_t N, int M, int64_t row0,
+                                           int m0, int lane) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int m = m0 + 2 * (lane & 3) + (r & 1);
+    const int64_t n = row0 + (lane >> 2) + 8 * (r >> 1);
+    if (m < M && n < N) y[(int64_t)m * N + n] = (uint16_t)float_to_bf16_bits(v[r]);
+  }
+}
+
+// Resident CTAs per SM that the register budget is for (two of 8 warps fit up to 32 batch rows, but only the balanced form,
+// whose loop over the groups makes the compiler generous, needs to be told with 4 tiles).
+template <int NT, int TPC, int W, bool SPLIT>
+constexpr int multi_ctas_per_sm() {
+  return W == 8 && (SPLIT ? NT <= 4 : NT <= 2 && TPC == 2) ? 2 : 1;
+}
+
+// SPLIT: the balanced form.  The (group of TPC tiles, step) units, group by group, are cut into gridDim.x equal ranges,
+// one per resident CTA; a group that several CTAs share leaves its sums in scratch for linear_multi_sum_kernel.
+template <int BITS, int NT, int TPC, int W, bool SPLIT>
+__global__ void __launch_bounds__(W * 32, (multi_ctas_per_sm<NT, TPC, W, SPLIT>())) linear_multi_kernel(
+    const uint32_t* __restrict__ packed, const uint16_t* __restrict__ cb, const uint16_t* __restrict__ x,
+    uint16_t* __restrict__ y, int64_t N, int64_t K, int M, float* __restrict__ scratch) {
   using G = MGeo<BITS>;
   using SM = MSmem<BITS, NT, TPC, W>;
   constexpr int kThreads = W * 32;
@@ -90,12 +110,14 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   const int wt = warp % TPC, group = warp / TPC;       // tile inside the CTA, K-group
   const int gtid = threadIdx.x - group * kGroupThreads;  // thread inside the K-group
   const int64_t tiles = (N + kTileRows - 1) / kTileRows;
-  const int64_t tile_id = (int64_t)blockIdx.x * TPC + wt;
-  const bool has_tile = tile_id < tiles;               // warp-uniform; such a warp still stages x and joins barriers
-  const int64_t row0 = tile_id * kTileRows;
   const int steps = (int)tuned_row_steps(K, BITS);
-  const uint4* __restrict__ tile =
-      reinterpret_cast<const uint4*>(packed) + (has_tile ? tile_id : 0) * (int64_t)steps * 64 + lane;
+  int64_t u0 = 0, u1 = 0, tg = blockIdx.x;   // SPLIT: units of this CTA; group of tiles
+  if constexpr (SPLIT) {
+    const int64_t units = (tiles + TPC - 1) / TPC * steps;
+    u0 = units * blockIdx.x / gridDim.x;
+    u1 = units * (blockIdx.x + 1) / gridDim.x;
+    tg = u0 / steps;
+  }
   unsigned char* const xgroup = xbase + group * 2 * SM::kBuf;
 
   // copy the activations under step s into buffer `buf` of this K-group (zeros past K; rows >= M are not touched:
@@ -112,13 +134,21 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
     cp_async_commit();
   };
 
+ do {   // one pass unless SPLIT
+  const int64_t base = tg * steps;
+  const int sa = SPLIT && u0 > base ? (int)(u0 - base) : 0, sb = SPLIT && u1 - base < steps ? (int)(u1 - base) : steps;
+  const int64_t tile_id = tg * TPC + wt;
+  const bool has_tile = tile_id < tiles;               // warp-uniform; such a warp still stages x and joins barriers
+  const int64_t row0 = tile_id * kTileRows;
+  const uint4* __restrict__ tile =
+      reinterpret_cast<const uint4*>(packed) + (has_tile ? tile_id : 0) * (int64_t)steps * 64 + lane;
   // ---- first loads: weights of this warp's first two steps, activations of the group's first step ----
   uint4 qa[2], qb[2];
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
-    const int s = group + d * kGroups;
+    const int s = sa + group + d * kGroups;
     qa[d] = qb[d] = make_uint4(0, 0, 0, 0);
-    if (has_tile && s < steps) {
+    if (has_tile && s < sb) {
       qa[d] = ldg_stream_u4(tile + (int64_t)s * 64);
       qb[d] = ldg_stream_u4(tile + (int64_t)s * 64 + 32);
     }
@@ -139,11 +169,12 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
     if constexpr (!SM::kTab) fg.init(cb + min(row0 + g, N - 1) * 16);
     fh.init(cb + min(row0 + g + 8, N - 1) * 16);
   }
+  if (SPLIT && base > u0) __syncthreads();   // the previous group's sums are read (they lie over the activations)
   if constexpr (SM::kTab) {
     // a thread takes a row and a low index: one fetch of the row's centroids, the 16 entries low + 16 high
     for (int it = threadIdx.x; it < TPC * 128; it += kThreads) {
       const int r8 = it & 7, low = (it >> 3) & 15, i = it >> 7;
-      const int64_t row = min(((int64_t)blockIdx.x * TPC + i) * kTileRows + r8, N - 1);
+      const int64_t row = min((tg * TPC + i) * kTileRows + r8, N - 1);
       const uint16_t* const crow = cb + row * 16;
       const uint4 ca = __ldg(reinterpret_cast<const uint4*>(crow)), cc = __ldg(reinterpret_cast<const uint4*>(crow) + 1);
       const uint32_t lo = __ldg(crow + low);
@@ -164,28 +195,30 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   // At b = 4, where the set-up of a CTA is long (its tables), the next kernel is released at once so that its CTAs
   // set up under this grid's MMAs; otherwise just before the partial sums are exchanged (measured, 4096 x 4096 M = 16:
   // b = 4 9.7 -> 8.3 us early, 8.7 late; b = 2 6.4 -> 6.3 / 6.5; 8192 x 8192 b = 2 M = 32 20.1 -> 20.1 / 19.5).
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if constexpr (BITS == 4) asm volatile("griddepcontrol.launch_dependents;");
-  if (group < steps) stage(group, 0);
+  if (!SPLIT || base <= u0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (BITS == 4) asm volatile("griddepcontrol.launch_dependents;");
+  }
+  if (sa + group < sb) stage(sa + group, 0);
 
   float acc[NT][4];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
 
-  for (int s0 = group; s0 < steps; s0 += 2 * kGroups) {   // uniform over the K-group
+  for (int s0 = sa + group; s0 < sb; s0 += 2 * kGroups) {   // uniform over the K-group
 #pragma unroll
    for (int buf = 0; buf < 2; ++buf) {                     // buffer index = parity of the group's step count
     const int s = s0 + buf * kGroups;
-    if (s >= steps) break;
+    if (s >= sb) break;
     cp_async_wait_all();
     group_barrier(group, kGroupThreads);   // x of step s is in place, and every warp of the group is done with step s - 2
-    if (s + kGroups < steps) stage(s + kGroups, buf ^ 1);
+    if (s + kGroups < sb) stage(s + kGroups, buf ^ 1);
     const unsigned char* const xs = xgroup + buf * SM::kBuf;
     if (has_tile) {
       const uint4 va = qa[buf], vb = qb[buf];
       const uint32_t wa[4] = {va.x, va.y, va.z, va.w};
       const uint32_t wb[4] = {vb.x, vb.y, vb.z, vb.w};
-      if (s + 2 * kGroups < steps) {   // refill for the step after next
+      if (s + 2 * kGroups < sb) {   // refill for the step after next
         qa[buf] = ldg_stream_u4(tile + (int64_t)(s + 2 * kGroups) * 64);
         qb[buf] = ldg_stream_u4(tile + (int64_t)(s + 2 * kGroups) * 64 + 32);
       }
@@ -241,7 +274,7 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
   }
 
   // ---- K-groups 1.. hand their partial sums to K-group 0, which adds and stores ----
-  asm volatile("griddepcontrol.launch_dependents;");
+  if (!SPLIT || base + steps >= u1) asm volatile("griddepcontrol.launch_dependents;");
   __syncthreads();   // every warp is done with the x buffers; `red` aliases them
   if (group > 0) {
 #pragma unroll
@@ -260,47 +293,122 @@ __global__ void __launch_bounds__(W * 32, (W == 8 && NT <= 2 && TPC == 2) ? 2 : 
             *reinterpret_cast<const float4*>(red + ((((gq - 1) * TPC + wt) * NT + nt) * 32 + lane) * 4);
         v[0] += o.x; v[1] += o.y; v[2] += o.z; v[3] += o.w;
       }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = nt * 8 + 2 * t + (r & 1);
-        const int64_t n = row0 + g + 8 * (r >> 1);
-        if (m < M && n < N) y[(int64_t)m * N + n] = (uint16_t)float_to_bf16_bits(v[r]);
-      }
+      if (!SPLIT || (sa == 0 && sb == steps)) store_sums(v, y, N, M, row0, nt * 8, lane);
+      else
+        reinterpret_cast<float4*>(scratch)[(((int64_t)blockIdx.x * 2 + (sa == 0 ? 1 : 0)) * (TPC * NT) + wt * NT + nt) * 32 +
+                                           lane] = make_float4(v[0], v[1], v[2], v[3]);
     }
   }
+ } while (SPLIT && ++tg * steps < u1);
 }
 
+// Block (c, tile of the group) adds the shares of group c where more than one CTA worked on it: slot [.][1] of the CTA
+// that started it, slot [.][0] of every later one, in that order.
+template <int BITS, int NT, int TPC>
+__global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* __restrict__ scratch,
+                                                                   uint16_t* __restrict__ y, int64_t N, int64_t K, int M,
+                                                                   int ctas) {
+  const int64_t steps = tuned_row_steps(K, BITS), groups = (N + TPC * kTileRows - 1) / (TPC * kTileRows);
+  const int64_t units = groups * steps;
+  // CTA c works on units [units c / ctas, units (c + 1) / ctas): unit u belongs to CTA ((u + 1) ctas - 1) / units
+  const int64_t first = (int64_t)blockIdx.x * steps, last = first + steps - 1;
+  const int64_t c0 = ((first + 1) * ctas - 1) / units, c1 = ((last + 1) * ctas - 1) / units;
+  if (c0 == c1) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  const float4* const src = reinterpret_cast<const float4*>(scratch) + (int64_t)blockIdx.y * NT * 32 + threadIdx.x;
+  constexpr int kSlot = TPC * NT * 32;
+  const float4 a = src[(c0 * 2 + 1) * kSlot];
+  float v[4] = {a.x, a.y, a.z, a.w};
+  for (int64_t c = c0 + 1; c <= c1; ++c) {
+    const float4 b = src[c * 2 * kSlot];
+    v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
+  }
+  store_sums(v, y, N, M, ((int64_t)blockIdx.x * TPC + blockIdx.y) * kTileRows, (threadIdx.x >> 5) * 8, threadIdx.x & 31);
+}
+
+// CTAs of the balanced form that fit an SM, asked from the runtime once per device.
+template <int BITS, int NT, int TPC, int W>
+int resident_ctas() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    constexpr int smem = MSmem<BITS, NT, TPC, W>::kTotal;
+    if (cudaFuncSetAttribute(linear_multi_kernel<BITS, NT, TPC, W, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, linear_multi_kernel<BITS, NT, TPC, W, true>, W * 32, smem) !=
+            cudaSuccess)
+      return 0;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+// A call; with `plan` set nothing is launched, and the shape of its CTA is put there.
+struct MultiCall {
+  const uint32_t* packed;
+  const uint16_t *cb, *x;
+  uint16_t* y;
+  int64_t N, K;
+  int M;
+  float* scratch;   // not null: the balanced form
+  MultiSplit* plan;
+  cudaStream_t s;
+};
+
 template <int BITS, int NT, int TPC, int W = 8>
-cudaError_t launch_nt(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N, int64_t K,
-                      int M, cudaStream_t s) {
+cudaError_t launch_nt(const MultiCall& c) {
   constexpr int smem = MSmem<BITS, NT, TPC, W>::kTotal;
+  const int64_t tiles = (c.N + kTileRows - 1) / kTileRows, groups = (tiles + TPC - 1) / TPC;
+  const DeviceInfo* di = device_info();
+  if (!di) return cudaErrorInvalidDevice;
+  const int slots = di->sm_count * resident_ctas<BITS, NT, TPC, W>();
+  if (slots <= 0) return cudaErrorInvalidConfiguration;
+  if (c.plan) {
+    c.plan->ctas = slots;
+    c.plan->tiles = TPC;
+    c.plan->groups = groups;
+    c.plan->scratch = (size_t)slots * 2 * TPC * NT * 512;
+    return cudaSuccess;
+  }
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !configured[dev]) {
-    cudaError_t e =
-        cudaFuncSetAttribute(linear_multi_kernel<BITS, NT, TPC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (dev >= 0 && dev < 64 && !configured[dev]) {   // (the balanced form: resident_ctas())
+    cudaError_t e = cudaFuncSetAttribute(linear_multi_kernel<BITS, NT, TPC, W, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  const int64_t tiles = (N + kTileRows - 1) / kTileRows;
-  const unsigned grid = (unsigned)((tiles + TPC - 1) / TPC);
+  const unsigned grid = c.scratch ? (unsigned)slots : (unsigned)groups;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(W * 32);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
+  cfg.stream = c.s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W>, packed, cb, x, y, N, K, M);
+  if (!c.scratch)
+    return cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, false>, c.packed, c.cb, c.x, c.y, c.N, c.K, c.M,
+                              c.scratch);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, true>, c.packed, c.cb, c.x, c.y, c.N, c.K,
+                                     c.M, c.scratch);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3((unsigned)groups, TPC);
+  cfg.blockDim = dim3(32 * NT);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, linear_multi_sum_kernel<BITS, NT, TPC>, (const float*)c.scratch, c.y, c.N, c.K, c.M, slots);
 }
 
 template <int BITS>
-cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
-                        int64_t K, int M, cudaStream_t s) {
+cudaError_t launch_bits(const MultiCall& c) {
+  const int64_t N = c.N, K = c.K;
+  const int M = c.M;
   // Tiles per CTA: 4 share the staged activations among more warps, 2 give twice as many CTAs.  Measured: 2 wins
   // when 4 would leave more than half of the SMs without a CTA, and for b = 2, 4 at up to 16 rows (two CTAs then fit an SM).
   const DeviceInfo* di = device_info();
@@ -313,41 +421,41 @@ cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16
   if (M <= 8) {
     // same shape of CTA for up to 8 batch rows (8192 x 28672, b = 1, M = 4: 35.0 -> 23.5 us; 8192 x 8192, b = 2,
     // M = 8: 12.7 -> 11.7 us)
-    if (!few && fits_one_wave) return launch_nt<BITS, 1, 4, 16>(packed, cb, x, y, N, K, M, s);
+    if (!few && fits_one_wave) return launch_nt<BITS, 1, 4, 16>(c);
     if constexpr (MSmem<BITS, 1, 2, 16>::kTotal <= kMaxSmem) {
-      if (few16) return launch_nt<BITS, 1, 2, 16>(packed, cb, x, y, N, K, M, s);
+      if (few16) return launch_nt<BITS, 1, 2, 16>(c);
     }
-    if (few || BITS != 1) return launch_nt<BITS, 1, 2>(packed, cb, x, y, N, K, M, s);
-    return launch_nt<BITS, 1, 4>(packed, cb, x, y, N, K, M, s);
+    if (few || BITS != 1) return launch_nt<BITS, 1, 2>(c);
+    return launch_nt<BITS, 1, 4>(c);
   }
   if (M <= 16) {
     // 4 tiles x 4 K-groups (16 warps) when that grid gives every SM at most one CTA: 8192 x 8192, b = 2, M = 16:
     // 16.1 -> 14.4 us; 8192 x 28672, M = 16: b = 1 47.9 -> 40.1 us, b = 4 85.2 -> 76.6 us
-    if (!few && fits_one_wave) return launch_nt<BITS, 2, 4, 16>(packed, cb, x, y, N, K, M, s);
+    if (!few && fits_one_wave) return launch_nt<BITS, 2, 4, 16>(c);
     if constexpr (MSmem<BITS, 2, 2, 16>::kTotal <= kMaxSmem) {
-      if (few16) return launch_nt<BITS, 2, 2, 16>(packed, cb, x, y, N, K, M, s);
+      if (few16) return launch_nt<BITS, 2, 2, 16>(c);
     }
-    if (few || BITS != 1) return launch_nt<BITS, 2, 2>(packed, cb, x, y, N, K, M, s);
-    return launch_nt<BITS, 2, 4>(packed, cb, x, y, N, K, M, s);
+    if (few || BITS != 1) return launch_nt<BITS, 2, 2>(c);
+    return launch_nt<BITS, 2, 4>(c);
   }
   if (M <= 32) {
     if constexpr (MSmem<BITS, 4, 2>::kTotal <= kMaxSmem) {
-      if (few) return launch_nt<BITS, 4, 2>(packed, cb, x, y, N, K, M, s);
+      if (few) return launch_nt<BITS, 4, 2>(c);
     }
     // when every SM gets at most one CTA anyway: 4 K-groups, i.e. 16 warps per CTA instead of 8 (8192 x 8192,
     // b = 2, M = 32: 22.6 -> 20.3 us; with more CTAs than SMs two 8-warp CTAs share an SM and that is faster)
     if constexpr (MSmem<BITS, 4, 4, 16>::kTotal <= kMaxSmem) {
-      if (fits_one_wave) return launch_nt<BITS, 4, 4, 16>(packed, cb, x, y, N, K, M, s);
+      if (fits_one_wave) return launch_nt<BITS, 4, 4, 16>(c);
     }
-    return launch_nt<BITS, 4, 4>(packed, cb, x, y, N, K, M, s);
+    return launch_nt<BITS, 4, 4>(c);
   }
   if constexpr (BITS == 1) {
     return cudaErrorInvalidValue;   // unreachable: b = 1 is launched in passes of at most 32 rows
   } else {
     if constexpr (MSmem<BITS, 8, 2>::kTotal <= kMaxSmem) {
-      if (few) return launch_nt<BITS, 8, 2>(packed, cb, x, y, N, K, M, s);
+      if (few) return launch_nt<BITS, 8, 2>(c);
     }
-    return launch_nt<BITS, 8, 4>(packed, cb, x, y, N, K, M, s);
+    return launch_nt<BITS, 8, 4>(c);
   }
 }
 
@@ -369,8 +477,28 @@ int linear_multi_min_rows(int bits, int64_t N) {
   return waves ? (bits == 2 ? 5 : 4) : 9;
 }
 
+static cudaError_t launch_multi(int bits, const MultiCall& c) {
+  return bits == 1 ? launch_bits<1>(c) : bits == 2 ? launch_bits<2>(c) : launch_bits<4>(c);
+}
+
+// Whether the balanced form is used (ctas > 0), and its scratch.  It saves the steps in which the last wave leaves CTA
+// slots empty and costs about 9000 clocks: the second kernel, and a CTA's start on one or two more groups.  A slot does
+// some 20 weights per clock and SM, 12 with more than 16 batch rows.  us per call, without / with: 8192 x 28672, M = 16
+// (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4, M = 16 32.5 / 25.6,
+// b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 16384 x 3072 18.0 / 19.4.
+MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
+  MultiSplit sp = {};
+  const DeviceInfo* di = device_info();
+  if (!di || M > linear_multi_rows_per_launch(bits)) return sp;
+  if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess) return {};
+  const int64_t steps = tuned_row_steps(K, bits), waves = (sp.groups + sp.ctas - 1) / sp.ctas;
+  const double saved = (double)(waves * sp.ctas - sp.groups) / sp.ctas * (double)steps;
+  const double step_clocks = (double)(sp.ctas / di->sm_count) * sp.tiles * (kTileRows * 512 / bits) / (M > 16 ? 12.0 : 20.0);
+  return saved * step_clocks > 9000.0 && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
+}
+
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
-                                int64_t K, int bits, int64_t M, cudaStream_t s) {
+                                int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s) {
   const int64_t per = linear_multi_rows_per_launch(bits);
   for (int64_t m0 = 0; m0 < M; m0 += per) {
     const int mc = (int)(M - m0 < per ? M - m0 : per);
@@ -378,9 +506,7 @@ cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, cons
     uint16_t* yp = y + m0 * N;
     cudaError_t e;
     if (mc < linear_multi_min_rows(bits, N)) e = launch_linear_tiled(packed, cb, xp, yp, N, K, bits, mc, s);   // a short tail
-    else if (bits == 1) e = launch_bits<1>(packed, cb, xp, yp, N, K, mc, s);
-    else if (bits == 2) e = launch_bits<2>(packed, cb, xp, yp, N, K, mc, s);
-    else e = launch_bits<4>(packed, cb, xp, yp, N, K, mc, s);
+    else e = launch_multi(bits, {packed, cb, xp, yp, N, K, mc, static_cast<float*>(scratch), nullptr, s});
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -27,10 +27,17 @@ int linear_split_ctas(int64_t N, int64_t K, int bits, int64_t M);
 size_t linear_split_scratch_bytes(int ctas);
 cudaError_t launch_linear_split(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, void* scratch, int ctas, cudaStream_t s);
+struct MultiSplit {     // the balanced form of the multi-tile kernel
+  int ctas;             // 0: not used
+  int tiles;            // tiles of a CTA
+  int64_t groups;       // groups of that many tiles
+  size_t scratch;
+};
+MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M);
 int linear_multi_rows_per_launch(int bits);
 int linear_multi_min_rows(int bits, int64_t N);   // smallest batch routed to the multi-tile kernel
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
-                                int64_t K, int bits, int64_t M, cudaStream_t s);
+                                int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s);   // scratch: balanced form
 bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M);   // kmq_linear's choice of the tcgen05 kernel
 int64_t linear_umma_rows_per_launch();
 int linear_umma_ksplit(int64_t N, int64_t K, int bits, int64_t batch);   // CTAs (cluster size) per 128-row block

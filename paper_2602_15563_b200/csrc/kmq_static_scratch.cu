@@ -47,7 +47,9 @@ extern "C" kmq_status kmq_linear_static_scratch(const uint32_t* packed, const ui
                                                 uint16_t* y, int64_t N, int64_t K, int bits, int64_t M, int layout,
                                                 void* stream) {
   // 0 both for shapes that need no scratch and for invalid arguments: kmq_linear sorts those out
-  const size_t need = kmq_workspace_bytes(N, K, bits, M, layout);
+  size_t need = kmq_workspace_bytes(N, K, bits, M, layout);
+  // only what cannot run without: the array is shared by all streams
+  if (need > 0) need = kmq::plan_linear(N, K, bits, M, layout, 0).workspace;
   if (need == 0) return kmq_linear(packed, codebooks, x, y, N, K, bits, M, layout, nullptr, 0, stream);
   if (need > kStaticScratchBytes) return KMQ_ERR_SCRATCH_LIMIT;
   cudaError_t err = cudaSuccess;

@@ -2,6 +2,7 @@
 tiles and row lengths."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import kmq_oracle as orc
 from paper_2602_15563_b200 import kmq
@@ -21,3 +22,21 @@ def test_half_tables(N, K, M):
     y = gu.gpu_linear(gu.gpu_pack(idx, 4, TUNED), cb, x, N, K, 4, TUNED)
     ratio = orc.check_linear(y, y_ref, s)
     assert ratio <= 1.0, f"error/tolerance = {ratio} [{kmq.kmq_linear_variant(N, K, 4, M, TUNED)}]"
+
+
+@pytest.mark.parametrize("bits,N,K,M", [(4, 10230, 8192, 16), (4, 8200, 28672, 5), (2, 10240, 8200, 32), (1, 9500, 20000, 9),
+                                        (4, 2050, 28680, 12), (2, 5130, 16400, 40)])
+def test_balanced_form(bits, N, K, M):
+    K = K // (32 // bits) * (32 // bits)
+    rng = np.random.default_rng(N + K + M)
+    idx, cb, x = random_layer(rng, N, K, bits, M)
+    y_ref, s = orc.linear_f64(orc.pack_canonical(idx, bits), cb, x, K, bits)
+    packed = gu.gpu_pack(idx, bits, TUNED)
+    y = gu.gpu_linear(packed, cb, x, N, K, bits, TUNED)
+    assert kmq.kmq_linear_variant(N, K, bits, M, TUNED).startswith("multi_balanced")
+    assert orc.check_linear(y, y_ref, s) <= 1.0
+    # without the scratch: the plain form
+    xd, cbd = gu.to_dev_u16(x), gu.to_dev_u16(cb)
+    yd = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    kmq.kmq_linear(packed, cbd, xd, yd, N, K, bits, M, None, 0, layout=TUNED)
+    assert orc.check_linear(yd.view(torch.int16).cpu().numpy().view(np.uint16), y_ref, s) <= 1.0
