@@ -26,6 +26,7 @@ constexpr int kWarps = 8;
 constexpr int kMinCtasPerSm = 3;   // register budget of the launch bounds
 constexpr int kThreads = kWarps * 32;
 constexpr int kRows = kTileRows;
+constexpr int kMaxCluster = 8;
 constexpr int kPairEntryStride = 256;   // b = 4 tables: entry e, half h, lane l at e * 256 + h * 128 + l * 4
 constexpr int kTableBytes4 = 256 * kPairEntryStride;
 
@@ -267,6 +268,37 @@ __device__ __forceinline__ void store_output(float v, uint16_t* __restrict__ y, 
   }
 }
 
+// One cluster of C CTAs per tile, each with a share of K: rank 0 adds the shares, handed to it through distributed shared
+// memory, in the order of the ranks.
+template <int BITS, int MMAX>
+__global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_cluster_kernel(const uint32_t* __restrict__ packed,
+                                                                    const uint16_t* __restrict__ cb,
+                                                                    const uint16_t* __restrict__ x,
+                                                                    uint16_t* __restrict__ y, int64_t N, int64_t K,
+                                                                    int M, int early, int C) {
+  __shared__ float shares[(kMaxCluster - 1) * kRows * 8];
+  // rank 0 has to be running before its shared memory is written: arrive now, wait before the write
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int steps = (int)tuned_row_steps(K, BITS), rank = (int)blockIdx.x % C;
+  const int64_t tile = blockIdx.x / C;
+  float v;
+  tile_segment<BITS, MMAX>(packed, cb, x, N, K, M, tile, steps * rank / C, steps * (rank + 1) / C, true, early != 0, v);
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank > 0 && threadIdx.x < kRows * 8) {
+    uint32_t dst;
+    const uint32_t own = (uint32_t)__cvta_generic_to_shared(shares + (rank - 1) * (kRows * 8) + threadIdx.x);
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"(own));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(v) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank == 0) {
+    if (threadIdx.x < kRows * 8)
+      for (int r = 1; r < C; ++r) v += shares[(r - 1) * (kRows * 8) + threadIdx.x];
+    store_output(v, y, N, M, tile * kRows);
+  }
+}
+
 // One CTA per tile.
 template <int BITS, int MMAX>
 __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_tiled_kernel(const uint32_t* __restrict__ packed,
@@ -357,6 +389,30 @@ bool early_trigger(int bits, int64_t tiles, int64_t steps, int sm_count) {
   return steps >= 16 && !(10 * tiles > 7 * two && tiles <= two);
 }
 
+// CTAs that share a tile, 1: linear_tiled_kernel.  In clocks, from sweeps at batch 1: a step takes a warp 1160 (2070 at
+// b = 1), the load it waits for included, and the SM 215 / 132 / 80 at b = 1 / 2 / 4; a cluster costs 1500 once (its
+// launch, two barriers, less overlap with the calls before and after).  More than two CTAs only while every SM has one at
+// most: beyond, clusters wait for room in one GPC (3072 x 8192, b = 2: 5.7 us, 5.1 by two, 7.0 by three).  us per call,
+// one / two / four CTAs per tile: 512 x 16384 b = 2 6.2 / 4.2 / 3.3, b = 4 11.0 / 6.5 / 4.2; 1024 x 8192 b = 4 5.9 / 4.1;
+// 3072 x 8192 b = 4 7.3 / 6.3; but 3072 x 3072 b = 2 2.7 / 3.4.
+int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di) {
+  if (!di) return 1;
+  const int64_t sms = di->sm_count, warp_step = bits == 1 ? 2070 : 1160, sm_step = bits == 1 ? 215 : bits == 2 ? 132 : 80;
+  int best = 1;
+  int64_t least = 0;
+  for (int c = 1; c <= kMaxCluster; c *= 2) {
+    if (c > 1 && (c > steps || tiles * c > (c == 2 ? kMinCtasPerSm : 1) * sms)) break;
+    const int64_t share = (steps + c - 1) / c;
+    const int64_t chain = (share + kWarps - 1) / kWarps * warp_step, issue = (tiles * c + sms - 1) / sms * share * sm_step;
+    const int64_t clocks = (chain > issue ? chain : issue) + (c > 1 ? 1500 : 0);
+    if (c == 1 || clocks + 300 < least) {
+      best = c;
+      least = clocks;
+    }
+  }
+  return best;
+}
+
 template <int BITS, int MMAX>
 cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                        int64_t K, int M, cudaStream_t s) {
@@ -367,6 +423,8 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     cudaError_t e =
         cudaFuncSetAttribute(linear_tiled_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(linear_cluster_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
@@ -375,13 +433,23 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const DeviceInfo* di = device_info();
   const int64_t steps = tuned_row_steps(K, BITS);
+  if (const int C = cluster_size(BITS, (N + kRows - 1) / kRows, steps, di); C > 1) {
+    cfg.gridDim.x *= C;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)C;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+    const int early = early_trigger(BITS, (N + kRows - 1) / kRows * C, steps / C, di->sm_count) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, linear_cluster_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M, early, C);
+  }
   const int early = di && early_trigger(BITS, (N + kRows - 1) / kRows, steps, di->sm_count) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, linear_tiled_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M, early);
 }
