@@ -15,6 +15,8 @@
 //   b = 2  the row's 4 centroids are the 8 source bytes of one PRMT; one PRMT yields two weights.
 //   b = 1  a shift (as a multiply on the FMA pipe) puts two index bits on bits 15 and 31, a sign-replicating PRMT
 //          spreads them over their half words and one LOP3 selects c0 or c1: bit copies of the stored centroids.
+#include <atomic>
+
 #include "kmq_common.cuh"
 #include "kmq_linear_variants.cuh"
 #include "kmq_mma_common.cuh"
@@ -395,13 +397,15 @@ bool early_trigger(int bits, int64_t tiles, int64_t steps, int sm_count) {
 // most: beyond, clusters wait for room in one GPC (3072 x 8192, b = 2: 5.7 us, 5.1 by two, 7.0 by three).  us per call,
 // one / two / four CTAs per tile: 512 x 16384 b = 2 6.2 / 4.2 / 3.3, b = 4 11.0 / 6.5 / 4.2; 1024 x 8192 b = 4 5.9 / 4.1;
 // 3072 x 8192 b = 4 7.3 / 6.3; but 3072 x 3072 b = 2 2.7 / 3.4.
-int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di) {
+// Two CTAs only while all clusters fit at once (`per_sm` CTAs of this instantiation on an SM): 2400 x 12000, b = 4, M = 3,
+// 300 CTAs on 296 slots: 11.7 us, 13.3 by two.
+int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di, int per_sm) {
   if (!di) return 1;
   const int64_t sms = di->sm_count, warp_step = bits == 1 ? 2070 : 1160, sm_step = bits == 1 ? 215 : bits == 2 ? 132 : 80;
   int best = 1;
   int64_t least = 0;
   for (int c = 1; c <= kMaxCluster; c *= 2) {
-    if (c > 1 && (c > steps || tiles * c > (c == 2 ? kMinCtasPerSm : 1) * sms)) break;
+    if (c > 1 && (c > steps || tiles * c > (c == 2 ? per_sm : 1) * sms)) break;
     const int64_t share = (steps + c - 1) / c;
     const int64_t chain = (share + kWarps - 1) / kWarps * warp_step, issue = (tiles * c + sms - 1) / sms * share * sm_step;
     const int64_t clocks = (chain > issue ? chain : issue) + (c > 1 ? 1500 : 0);
@@ -411,6 +415,24 @@ int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di) {
     }
   }
   return best;
+}
+
+// CTAs of linear_cluster_kernel<BITS, MMAX> that fit one SM, asked from the runtime once per device and instantiation.
+template <int BITS, int MMAX>
+int cluster_ctas_per_sm() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    constexpr int smem = TSmem<BITS, MMAX>::kTotal;
+    if (cudaFuncSetAttribute(linear_cluster_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, linear_cluster_kernel<BITS, MMAX>, kThreads, smem) != cudaSuccess)
+      return 0;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
 }
 
 template <int BITS, int MMAX>
@@ -423,8 +445,6 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     cudaError_t e =
         cudaFuncSetAttribute(linear_tiled_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(linear_cluster_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
@@ -440,7 +460,7 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   cfg.numAttrs = 1;
   const DeviceInfo* di = device_info();
   const int64_t steps = tuned_row_steps(K, BITS);
-  if (const int C = cluster_size(BITS, (N + kRows - 1) / kRows, steps, di); C > 1) {
+  if (const int C = cluster_size(BITS, (N + kRows - 1) / kRows, steps, di, cluster_ctas_per_sm<BITS, MMAX>()); C > 1) {
     cfg.gridDim.x *= C;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)C;
