@@ -1,4 +1,4 @@
-// kmq_linear on the tuned (tile-major) layout for batches of up to 64 rows per launch (chosen from 4, 5 or 9 rows
+// kmq_linear on the tuned (tile-major) layout for batches of up to 64 rows per launch (chosen from 2 to 9 rows
 // on, see linear_multi_min_rows): the tiles of a CTA share the staged activations, and the decode of a weight
 // fragment is paid once and reused by up to 8 MMAs (one per group of 8 batch rows).
 //
@@ -464,17 +464,33 @@ cudaError_t launch_bits(const MultiCall& c) {
 // Batch rows per launch of the multi-tile kernel: 64, or 32 for b = 1 (its x buffers are twice as large).
 int linear_multi_rows_per_launch(int bits) { return bits == 1 ? 32 : 64; }
 
-// Smallest batch that goes to the multi-tile kernel.  The GEMV kernel stages the activations of a step once per
-// warp and tile; at b = 1 a step spans 512 activations per batch row against 1 KB of packed words, so from 3 batch
-// rows on sharing the staged activations among the tiles of a CTA wins (8192 x 28672: 33 -> 23 us at M = 3,
-// 88 -> 25 us at M = 8), from 2 rows on when the GEMV grid would not fit the SMs in one wave of CTAs.  At b = 2, 4 it
-// only wins on such shapes, from 5 and 4 rows on.
-int linear_multi_min_rows(int bits, int64_t N) {
+// Smallest batch that goes to the multi-tile kernel.  The GEMV kernel stages the activations once per tile, here the tiles
+// of a CTA share them; but its grid is finer, and it shares K among a cluster.  us per call, GEMV / multi-tile:
+//   b = 1  more than three tiles per SM: 2 rows on.  Otherwise up to 4 rows stay (1024 x 8192, M = 3 3.5 / 5.4; 6144 x 8192,
+//          M = 4 8.4 / 9.8) except on long rows (2048 x 28672, M = 3 11.2 / 10.6) and on few steps that two CTAs of one SM
+//          and one of another share badly (3072 x 3072, M = 3 3.6 / 3.4).
+//   b = 2  waves: 5 rows on, on long rows 2 (8192 x 28672, M = 2 34.0 / 30.0).  One wave: 9, on long rows 2 where the
+//          GEMV kernel does not use clusters (4096 x 9216, M = 2 9.2 / 7.1, M = 8 11.8 / 8.1), 5 where it uses two CTAs on
+//          a full machine (3072 x 16384, M = 4 9.6 / 10.4, M = 8 11.5 / 10.9).
+//   b = 4  from 3 rows on the GEMV kernel's tables leave room for two CTAs per SM: 3 where the tiles do not fit these slots
+//          (6144 x 4096, M = 3 9.1 / 8.3, M = 8 11.1 / 8.7) and on long rows (3072 x 16384, M = 4 16.2 / 15.0); 7 on
+//          medium ones (4096 x 4096, M = 8 6.3 / 5.6; 3072 x 8192 9.9 / 8.8); else 9.
+int linear_multi_min_rows(int bits, int64_t N, int64_t K) {
   const DeviceInfo* di = device_info();
-  const int64_t tiles = (N + kTileRows - 1) / kTileRows;
-  const bool waves = di && tiles > (int64_t)di->sm_count * 3;
-  if (bits == 1) return waves ? 2 : 3;
-  return waves ? (bits == 2 ? 5 : 4) : 9;
+  const int64_t sms = di ? di->sm_count : 148, tiles = (N + kTileRows - 1) / kTileRows, steps = tuned_row_steps(K, bits);
+  const bool waves = tiles > sms * 3;
+  if (bits == 1) {
+    if (waves) return 2;
+    return steps > 32 || (steps < 8 && tiles > sms && 2 * tiles <= 3 * sms) ? 3 : 5;
+  }
+  if (bits == 2) {
+    if (waves) return steps > 64 ? 2 : 5;
+    if (steps <= 32 || 2 * tiles <= sms || tiles > 2 * sms) return 9;
+    return tiles > sms && 2 * tiles <= 3 * sms ? 5 : 2;
+  }
+  if (tiles > 2 * sms) return 3;
+  if (tiles <= sms || steps < 32) return 9;
+  return steps > 64 ? 3 : 7;
 }
 
 static cudaError_t launch_multi(int bits, const MultiCall& c) {
@@ -505,7 +521,7 @@ cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, cons
     const uint16_t* xp = x + m0 * K;
     uint16_t* yp = y + m0 * N;
     cudaError_t e;
-    if (mc < linear_multi_min_rows(bits, N)) e = launch_linear_tiled(packed, cb, xp, yp, N, K, bits, mc, s);   // a short tail
+    if (mc < linear_multi_min_rows(bits, N, K)) e = launch_linear_tiled(packed, cb, xp, yp, N, K, bits, mc, s);   // a short tail
     else e = launch_multi(bits, {packed, cb, xp, yp, N, K, mc, static_cast<float*>(scratch), nullptr, s});
     if (e != cudaSuccess) return e;
   }

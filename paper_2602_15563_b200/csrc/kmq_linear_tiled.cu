@@ -481,7 +481,7 @@ cudaError_t launch_bits(const uint32_t* packed, const uint16_t* cb, const uint16
   if (M == 2) return launch_one<BITS, 2>(packed, cb, x, y, N, K, M, s);
   if (M <= 4) return launch_one<BITS, 4>(packed, cb, x, y, N, K, M, s);
   if constexpr (BITS == 1) {
-    return cudaErrorInvalidValue;   // unreachable: b = 1 goes to the multi-tile kernel from 4 batch rows on
+    return cudaErrorInvalidValue;   // unreachable: b = 1 goes to the multi-tile kernel from 5 batch rows on
   } else {
     return launch_one<BITS, 8>(packed, cb, x, y, N, K, M, s);
   }
@@ -589,7 +589,7 @@ int split_ctas_per_sm_bits(int64_t M) {
 
 int linear_split_ctas(int64_t N, int64_t K, int bits, int64_t M) {
   const DeviceInfo* di = device_info();
-  if (!di || M > 4 || M >= linear_multi_min_rows(bits, N)) return 0;
+  if (!di || M > 4 || M >= linear_multi_min_rows(bits, N, K)) return 0;
   // one CTA per resident slot of the instantiation that will run, so that there is no second wave
   const int per_sm = bits == 1 ? split_ctas_per_sm_bits<1>(M) : bits == 2 ? split_ctas_per_sm_bits<2>(M)
                                                                             : split_ctas_per_sm_bits<4>(M);
