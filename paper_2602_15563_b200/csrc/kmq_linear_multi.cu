@@ -498,18 +498,22 @@ static cudaError_t launch_multi(int bits, const MultiCall& c) {
 }
 
 // Whether the balanced form is used (ctas > 0), and its scratch.  It saves the steps in which the last wave leaves CTA
-// slots empty and costs about 9000 clocks: the second kernel, and a CTA's start on one or two more groups.  A slot does
-// some 20 weights per clock and SM, 12 with more than 16 batch rows.  us per call, without / with: 8192 x 28672, M = 16
-// (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4, M = 16 32.5 / 25.6,
-// b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 16384 x 3072 18.0 / 19.4.
+// slots empty and costs about 9000 clocks: the second kernel, and a CTA's start on one or two more groups.  An SM does
+// some 20 weights per clock (24 at b = 2), 27 up to 8 batch rows, 12 with more than 16.  us per call, without / with:
+// 8192 x 28672, M = 16 (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4,
+// M = 16 32.5 / 25.6, b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 12288 x 4096, b = 2, M = 12
+// 12.9 / 13.5.
 MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
   MultiSplit sp = {};
   const DeviceInfo* di = device_info();
   if (!di || M > linear_multi_rows_per_launch(bits)) return sp;
   if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess) return {};
-  const int64_t steps = tuned_row_steps(K, bits), waves = (sp.groups + sp.ctas - 1) / sp.ctas;
-  const double saved = (double)(waves * sp.ctas - sp.groups) / sp.ctas * (double)steps;
-  const double step_clocks = (double)(sp.ctas / di->sm_count) * sp.tiles * (kTileRows * 512 / bits) / (M > 16 ? 12.0 : 20.0);
+  const int64_t steps = tuned_row_steps(K, bits);
+  // CTAs that have an SM to themselves run as fast as the SM lets them: then it is the SMs that are empty, not the slots
+  const int64_t slots = sp.groups <= di->sm_count ? di->sm_count : sp.ctas, waves = (sp.groups + slots - 1) / slots;
+  const double saved = (double)(waves * slots - sp.groups) / slots * (double)steps;
+  const double step_clocks =
+      (double)(slots / di->sm_count) * sp.tiles * (kTileRows * 512 / bits) / (M > 16 ? 12.0 : M <= 8 ? 27.0 : bits == 2 ? 24.0 : 20.0);
   return saved * step_clocks > 9000.0 && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
 }
 

@@ -393,7 +393,7 @@ bool early_trigger(int bits, int64_t tiles, int64_t steps, int sm_count) {
 
 // CTAs that share a tile, 1: linear_tiled_kernel.  In clocks, from sweeps at batch 1: a step takes a warp 1160 (2070 at
 // b = 1), the load it waits for included, and the SM 215 / 132 / 80 at b = 1 / 2 / 4; a cluster costs 1500 once (its
-// launch, two barriers, less overlap with the calls before and after).  More than two CTAs only while every SM has one at
+// launch, two barriers, less overlap with the calls before and after), 2400 where it alone puts two CTAs on an SM.  More than two CTAs only while every SM has one at
 // most: beyond, clusters wait for room in one GPC (3072 x 8192, b = 2: 5.7 us, 5.1 by two, 7.0 by three).  us per call,
 // one / two / four CTAs per tile: 512 x 16384 b = 2 6.2 / 4.2 / 3.3, b = 4 11.0 / 6.5 / 4.2; 1024 x 8192 b = 4 5.9 / 4.1;
 // 3072 x 8192 b = 4 7.3 / 6.3; but 3072 x 3072 b = 2 2.7 / 3.4.
@@ -408,7 +408,7 @@ int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di, i
     if (c > 1 && (c > steps || tiles * c > (c == 2 ? per_sm : 1) * sms)) break;
     const int64_t share = (steps + c - 1) / c;
     const int64_t chain = (share + kWarps - 1) / kWarps * warp_step, issue = (tiles * c + sms - 1) / sms * share * sm_step;
-    const int64_t clocks = (chain > issue ? chain : issue) + (c > 1 ? 1500 : 0);
+    const int64_t clocks = (chain > issue ? chain : issue) + (c == 1 ? 0 : tiles <= sms && tiles * c > sms ? 2400 : 1500);
     if (c == 1 || clocks + 300 < least) {
       best = c;
       least = clocks;
