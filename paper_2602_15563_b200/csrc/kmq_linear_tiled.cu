@@ -86,7 +86,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int64_t row0 = tile_id * kRows;
-  const int steps = (int)tuned_row_steps(K, BITS);
+  const int steps = (int)((uint32_t)(K + G::kStepK - 1) / G::kStepK);
   // step s of this tile: 64 16-byte units, unit h * 32 + lane = row (g + 8h), chunk t
   const uint4* __restrict__ tile = reinterpret_cast<const uint4*>(packed) + tile_id * steps * 64 + lane;
   __syncthreads();   // a previous segment's readers of the tables and of `red` are done
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_tiled_kernel(c
                                                                     const uint16_t* __restrict__ x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, int early) {
-  const int steps = (int)tuned_row_steps(K, BITS);
+  const int steps = (int)((uint32_t)(K + TGeo<BITS>::kStepK - 1) / TGeo<BITS>::kStepK);
   const int64_t row0 = (int64_t)blockIdx.x * kRows;
   float v;
   tile_segment<BITS, MMAX>(packed, cb, x, N, K, M, blockIdx.x, 0, steps, true, early != 0, v);
@@ -393,12 +393,12 @@ bool early_trigger(int bits, int64_t tiles, int64_t steps, int sm_count) {
 
 // CTAs that share a tile, 1: linear_tiled_kernel.  In clocks, from sweeps at batch 1: a step takes a warp 1160 (2070 at
 // b = 1), the load it waits for included, and the SM 215 / 132 / 80 at b = 1 / 2 / 4; a cluster costs 1500 once (its
-// launch, two barriers, less overlap with the calls before and after), 2400 where it alone puts two CTAs on an SM.  More than two CTAs only while every SM has one at
-// most: beyond, clusters wait for room in one GPC (3072 x 8192, b = 2: 5.7 us, 5.1 by two, 7.0 by three).  us per call,
-// one / two / four CTAs per tile: 512 x 16384 b = 2 6.2 / 4.2 / 3.3, b = 4 11.0 / 6.5 / 4.2; 1024 x 8192 b = 4 5.9 / 4.1;
-// 3072 x 8192 b = 4 7.3 / 6.3; but 3072 x 3072 b = 2 2.7 / 3.4.
-// Two CTAs only while all clusters fit at once (`per_sm` CTAs of this instantiation on an SM): 2400 x 12000, b = 4, M = 3,
-// 300 CTAs on 296 slots: 11.7 us, 13.3 by two.
+// launch, two barriers, less overlap with the calls before and after), 2400 where it alone puts two CTAs on an SM.  Two
+// CTAs only while all clusters fit at once (`per_sm` CTAs of this instantiation on an SM; 2400 x 12000, b = 4, M = 3, 300
+// CTAs on 296 slots: 11.7 us, 13.3 by two), more only while every SM has one at most: beyond, clusters wait for room in one
+// GPC (3072 x 8192, b = 2: 5.7 us, 5.1 by two, 7.0 by three).  us per call, one / two / four CTAs per tile: 512 x 16384
+// b = 2 6.2 / 4.2 / 3.3, b = 4 11.0 / 6.5 / 4.2; 1024 x 8192 b = 4 5.9 / 4.1; 3072 x 8192 b = 4 7.3 / 6.3; but 3072 x 3072
+// b = 2 2.7 / 3.4.
 int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di, int per_sm) {
   if (!di) return 1;
   const int64_t sms = di->sm_count, warp_step = bits == 1 ? 2070 : 1160, sm_step = bits == 1 ? 215 : bits == 2 ? 132 : 80;
