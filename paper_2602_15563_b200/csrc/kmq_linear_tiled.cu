@@ -526,8 +526,7 @@ cudaError_t launch_split_bits(const uint32_t* packed, const uint16_t* cb, const 
                               int64_t K, int M, float* scratch, int ctas, cudaStream_t s) {
   if (M == 1) return launch_split_one<BITS, 1>(packed, cb, x, y, N, K, M, scratch, ctas, s);
   if (M == 2) return launch_split_one<BITS, 2>(packed, cb, x, y, N, K, M, scratch, ctas, s);
-  if (M <= 4) return launch_split_one<BITS, 4>(packed, cb, x, y, N, K, M, scratch, ctas, s);
-  return cudaErrorInvalidValue;   // unreachable: with more tiles than CTA slots, 5 rows and more go to the multi-tile kernel
+  return cudaErrorInvalidValue;   // unreachable: with more tiles than CTA slots, 3 rows and more go to the multi-tile kernel
 }
 
 }  // namespace
@@ -582,14 +581,14 @@ int split_ctas_per_sm() {
 
 template <int BITS>
 int split_ctas_per_sm_bits(int64_t M) {
-  return M == 1 ? split_ctas_per_sm<BITS, 1>() : M == 2 ? split_ctas_per_sm<BITS, 2>() : split_ctas_per_sm<BITS, 4>();
+  return M == 1 ? split_ctas_per_sm<BITS, 1>() : split_ctas_per_sm<BITS, 2>();
 }
 
 }  // namespace
 
 int linear_split_ctas(int64_t N, int64_t K, int bits, int64_t M) {
   const DeviceInfo* di = device_info();
-  if (!di || M > 4 || M >= linear_multi_min_rows(bits, N, K)) return 0;
+  if (!di || M > 2 || M >= linear_multi_min_rows(bits, N, K)) return 0;
   // one CTA per resident slot of the instantiation that will run, so that there is no second wave
   const int per_sm = bits == 1 ? split_ctas_per_sm_bits<1>(M) : bits == 2 ? split_ctas_per_sm_bits<2>(M)
                                                                             : split_ctas_per_sm_bits<4>(M);

@@ -12,7 +12,7 @@ enum LinearVariant : int {
                          // activations, one decode feeds up to 8 MMAs
   kVariantUmma = 5,      // tuned layout, M > 32 and enough 128-row blocks to fill the SMs: tcgen05.mma, weights
                          // dequantised into tensor memory
-  kVariantSplit = 4,     // tuned layout, M <= 8, more tiles than resident CTAs: equal step ranges + fix-up (scratch)
+  kVariantSplit = 4,     // tuned layout, M <= 2, more tiles than resident CTAs: equal step ranges + fix-up (scratch)
   kVariantLut = 6,       // table layout, b = 1, 2: activation tables in shared memory, one lookup per 8 weights (scratch)
   kVariantUnsupported = 7,
 };
