@@ -3,6 +3,8 @@
 // its own start (4096 x 4096, b = 1, M = 1, 8 KB each way: 21.7 us with two copies, 13 us of it not the layer).  The
 // kernels read or write the pinned memory over the bus directly; under programmatic dependent launch the layer's own
 // kernel sets up (packed indices, tables) while the activations arrive.
+#include <cuda.h>
+
 #include "kmq_common.cuh"
 
 namespace kmq {
@@ -25,16 +27,31 @@ __global__ void __launch_bounds__(kCopyThreads) host_copy_kernel(void* __restric
 }  // namespace
 
 // The device's address of pinned host memory that a kernel can copy with 16-byte accesses; nullptr where the memory is
-// pageable or unaligned, or the copy is large enough for the copy engine's bandwidth to matter.
+// pageable or unaligned, or the copy is large enough for the copy engine's bandwidth to matter.  The whole copy has to lie
+// in one allocation or registration: of a buffer that is pinned in part a kernel would touch unmapped addresses, while
+// cudaMemcpyAsync sees the range and refuses.  (One driver call, 35 ns; cudaPointerGetAttributes, which knows no ranges,
+// takes 56.)
 void* host_copy_address(const void* host, size_t bytes) {
   constexpr size_t kMost = 256 * 1024;
   if (bytes > kMost || (reinterpret_cast<uintptr_t>(host) & 15u) != 0) return nullptr;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
-    cudaGetLastError();   // not an address this runtime knows: an ordinary pageable one
-    return nullptr;
-  }
-  return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+  static const auto get_attributes = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr)>(p);
+  }();
+  if (!get_attributes) return nullptr;
+  CUmemorytype type = (CUmemorytype)0;   // all of these stay 0 for memory that is not pinned
+  CUdeviceptr device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* where[] = {&type, &device, &start, &size};
+  if (get_attributes(4, what, where, reinterpret_cast<CUdeviceptr>(host)) != CUDA_SUCCESS) return nullptr;
+  const bool inside = device >= start && device - start <= size && bytes <= size - (device - start);
+  return type == CU_MEMORYTYPE_HOST && inside ? reinterpret_cast<void*>(device) : nullptr;
 }
 
 cudaError_t launch_host_copy(void* dst, const void* src, size_t bytes, cudaStream_t s) {
