@@ -127,7 +127,7 @@ __device__ __forceinline__ float chunk_sum(uint32_t unit_addr, int lane, const u
 template <int BITS, int NL>
 __global__ void __launch_bounds__(BGeo<BITS, NL>::kWarps * 32, 1)
     block_lut_kernel(const unsigned char* __restrict__ tab, const uint16_t* __restrict__ codebook,
-                     const uint16_t* __restrict__ x, uint16_t* __restrict__ y, float* __restrict__ scratch, int64_t N,
+                     const uint16_t* x, uint16_t* __restrict__ y, float* __restrict__ scratch, int64_t N,
                      int64_t K, int slices, int row_blocks, unsigned int* __restrict__ err) {
   using G = BGeo<BITS, NL>;
   constexpr int S = G::kStagesPerWarp, UB = G::kUnit, GW = 8 / BITS;   // GW = weights per group
@@ -207,12 +207,12 @@ __global__ void __launch_bounds__(BGeo<BITS, NL>::kWarps * 32, 1)
       const int64_t k0 = ((int64_t)(chunk0 + (item >> 4)) * 32 + lane) * GW;
       xv[u] = make_uint4(0, 0, 0, 0);
       if (item < kItems && k0 < K) {
-        if constexpr (BITS == 1) xv[u] = __ldg(reinterpret_cast<const uint4*>(x + k0));
+        if constexpr (BITS == 1) xv[u] = ld_input_u4(x + k0);
         else if constexpr (BITS == 2) {
-          const uint2 t = __ldg(reinterpret_cast<const uint2*>(x + k0));
+          const uint2 t = ld_input_u2(x + k0);
           xv[u].x = t.x;
           xv[u].y = t.y;
-        } else xv[u].x = __ldg(reinterpret_cast<const uint32_t*>(x + k0));
+        } else xv[u].x = ld_input_u32(x + k0);
       }
     }
 #pragma unroll
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(BGeo<BITS, NL>::kWarps * 32, 1)
 constexpr int kFinWarps = 8;
 
 __global__ void __launch_bounds__(kFinWarps * 32)
-    block_lut_finish_kernel(const float* __restrict__ scratch, uint16_t* __restrict__ y, int64_t N, int slices) {
+    block_lut_finish_kernel(const float* scratch, uint16_t* __restrict__ y, int64_t N, int slices) {
   __shared__ float part[kFinWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t rows_pad = table_tiles(N) * 16;

@@ -13,15 +13,14 @@ namespace {
 constexpr int kCopyThreads = 256;
 
 // 16 bytes per thread and round; the last bytes two at a time (bf16 values)
-__global__ void __launch_bounds__(kCopyThreads) host_copy_kernel(void* __restrict__ dst, const void* __restrict__ src,
-                                                                 int64_t bytes) {
+__global__ void __launch_bounds__(kCopyThreads) host_copy_kernel(void* dst, const void* src, int64_t bytes) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
   const int64_t stride = (int64_t)gridDim.x * kCopyThreads, first = (int64_t)blockIdx.x * kCopyThreads + threadIdx.x;
   for (int64_t i = first; i < bytes / 16; i += stride)
-    static_cast<uint4*>(dst)[i] = static_cast<const uint4*>(src)[i];
+    static_cast<uint4*>(dst)[i] = ld_input_u4(static_cast<const uint4*>(src) + i);
   const int64_t tail = bytes / 16 * 8;
-  if (tail + first < bytes / 2) static_cast<uint16_t*>(dst)[tail + first] = static_cast<const uint16_t*>(src)[tail + first];
+  if (tail + first < bytes / 2) static_cast<uint16_t*>(dst)[tail + first] = ld_input_u16(static_cast<const uint16_t*>(src) + tail + first);
 }
 
 }  // namespace

@@ -125,7 +125,7 @@ __host__ __device__ inline size_t lut_scratch_floats(int slices, int classes, in
 template <int BITS, int NL>
 __global__ void __launch_bounds__(LutGeo<BITS, NL>::kWarps * 32, 1)
     linear_lut_kernel(const unsigned char* __restrict__ packed, const uint16_t* __restrict__ cb,
-                      const uint16_t* __restrict__ x, uint16_t* __restrict__ y, float* __restrict__ scratch, int64_t N,
+                      const uint16_t* x, uint16_t* __restrict__ y, float* __restrict__ scratch, int64_t N,
                       int64_t K, int slices, int row_blocks, unsigned int* __restrict__ err, int in_cluster) {
   using G = LutGeo<BITS, NL>;
   constexpr int CL = G::kClasses, S = G::kStages, P = G::kPieces, PC = G::kPieceChunks, TPR = G::kTasksPerRound;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(LutGeo<BITS, NL>::kWarps * 32, 1)
       const int item = warp + u * nwarps;
       const int64_t k0 = ((int64_t)(chunk0 + (item >> 4)) * 32 + lane) * 8;
       xv[u] = make_uint4(0, 0, 0, 0);
-      if (item < kItems && k0 < K) xv[u] = __ldg(reinterpret_cast<const uint4*>(x + k0));
+      if (item < kItems && k0 < K) xv[u] = ld_input_u4(x + k0);
     }
 #pragma unroll
     for (int u = 0; u < kMaxPerWarp; ++u) {
@@ -419,7 +419,7 @@ constexpr int kFinWarps = 8;
 
 template <int BITS>
 __global__ void __launch_bounds__(kFinWarps * 32)
-    linear_lut_finish_kernel(const float* __restrict__ scratch, const uint16_t* __restrict__ cb,
+    linear_lut_finish_kernel(const float* scratch, const uint16_t* __restrict__ cb,
                              uint16_t* __restrict__ y, int64_t N, int slices) {
   constexpr int CL = BITS == 1 ? 1 : 3;
   __shared__ float part[kFinWarps][CL + 1][32];

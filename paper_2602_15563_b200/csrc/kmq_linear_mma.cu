@@ -49,15 +49,15 @@ constexpr int smem_bytes() {
 // feeds to MMA (j, q), in the order the weight decode produces them.
 // ---------------------------------------------------------------------------
 template <int BITS>
-__device__ __forceinline__ void stage_block(const uint16_t* __restrict__ xrow, int64_t k0, bool valid,
+__device__ __forceinline__ void stage_block(const uint16_t* xrow, int64_t k0, bool valid,
                                             unsigned char* dst) {
   // dst: unit [slot = j*kMmaPerWord][t] of this batch row; consecutive MMAs of the word are 32 bytes apart
   constexpr int Q = Geo<BITS>::kMmaPerWord;
   if constexpr (BITS == 2) {
     uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (valid) {
-      const uint4 v0 = __ldg(reinterpret_cast<const uint4*>(xrow + k0));
-      const uint4 v1 = __ldg(reinterpret_cast<const uint4*>(xrow + k0 + 8));
+      const uint4 v0 = ld_input_u4(xrow + k0);
+      const uint4 v1 = ld_input_u4(xrow + k0 + 8);
       r[0] = v0.x; r[1] = v0.y; r[2] = v0.z; r[3] = v0.w; r[4] = v1.x; r[5] = v1.y; r[6] = v1.z; r[7] = v1.w;
     }
     // MMA q takes weights (q, q+4 | q+8, q+12) of the 16-weight word
@@ -75,7 +75,7 @@ __device__ __forceinline__ void stage_block(const uint16_t* __restrict__ xrow, i
     if (valid) {
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        const uint4 u = __ldg(reinterpret_cast<const uint4*>(xrow + k0 + 8 * v));
+        const uint4 u = ld_input_u4(xrow + k0 + 8 * v);
         r[4 * v] = u.x; r[4 * v + 1] = u.y; r[4 * v + 2] = u.z; r[4 * v + 3] = u.w;
       }
     }
@@ -88,7 +88,7 @@ __device__ __forceinline__ void stage_block(const uint16_t* __restrict__ xrow, i
 }
 
 template <int BITS>
-__device__ __forceinline__ void stage_step(const uint16_t* __restrict__ x, int64_t K, int M, int64_t step,
+__device__ __forceinline__ void stage_step(const uint16_t* x, int64_t K, int M, int64_t step,
                                            unsigned char* xs_warp, int lane) {
   using G = Geo<BITS>;
   const int blk = lane & 15;                 // 16 word blocks per batch row: chunk t = blk / 4, word j = blk % 4
@@ -102,7 +102,7 @@ __device__ __forceinline__ void stage_step(const uint16_t* __restrict__ x, int64
 template <int BITS, int MMAX>
 __global__ void __launch_bounds__(kThreads) linear_mma_kernel(const uint32_t* __restrict__ packed,
                                                               const uint16_t* __restrict__ cb,
-                                                              const uint16_t* __restrict__ x, uint16_t* __restrict__ y,
+                                                              const uint16_t* x, uint16_t* __restrict__ y,
                                                               int64_t N, int64_t K, int M) {
   using G = Geo<BITS>;
   constexpr int Q = G::kMmaPerWord;

@@ -94,7 +94,7 @@ constexpr int multi_ctas_per_sm() {
 // one per resident CTA; a group that several CTAs share leaves its sums in scratch for linear_multi_sum_kernel.
 template <int BITS, int NT, int TPC, int W, bool SPLIT>
 __global__ void __launch_bounds__(W * 32, (multi_ctas_per_sm<NT, TPC, W, SPLIT>())) linear_multi_kernel(
-    const uint32_t* __restrict__ packed, const uint16_t* __restrict__ cb, const uint16_t* __restrict__ x,
+    const uint32_t* __restrict__ packed, const uint16_t* __restrict__ cb, const uint16_t* x,
     uint16_t* __restrict__ y, int64_t N, int64_t K, int M, float* __restrict__ scratch) {
   using G = MGeo<BITS>;
   using SM = MSmem<BITS, NT, TPC, W>;
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(W * 32, (multi_ctas_per_sm<NT, TPC, W, SPLIT>(
 // Block (c, tile of the group) adds the shares of group c where more than one CTA worked on it: slot [.][1] of the CTA
 // that started it, slot [.][0] of every later one, in that order.
 template <int BITS, int NT, int TPC>
-__global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* __restrict__ scratch,
+__global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* scratch,
                                                                    uint16_t* __restrict__ y, int64_t N, int64_t K, int M,
                                                                    int ctas) {
   const int64_t steps = tuned_row_steps(K, BITS), groups = (N + TPC * kTileRows - 1) / (TPC * kTileRows);
@@ -318,11 +318,12 @@ __global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* 
   asm volatile("griddepcontrol.launch_dependents;");
   const float4* const src = reinterpret_cast<const float4*>(scratch) + (int64_t)blockIdx.y * NT * 32 + threadIdx.x;
   constexpr int kSlot = TPC * NT * 32;
-  const float4 a = src[(c0 * 2 + 1) * kSlot];
-  float v[4] = {a.x, a.y, a.z, a.w};
+  float v[4];
+  const uint4 a = ld_input_u4(src + (c0 * 2 + 1) * kSlot);
+  v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y); v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
   for (int64_t c = c0 + 1; c <= c1; ++c) {
-    const float4 b = src[c * 2 * kSlot];
-    v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
+    const uint4 b = ld_input_u4(src + c * 2 * kSlot);
+    v[0] += __uint_as_float(b.x); v[1] += __uint_as_float(b.y); v[2] += __uint_as_float(b.z); v[3] += __uint_as_float(b.w);
   }
   store_sums(v, y, N, M, ((int64_t)blockIdx.x * TPC + blockIdx.y) * kTileRows, (threadIdx.x >> 5) * 8, threadIdx.x & 31);
 }

@@ -66,7 +66,7 @@ __device__ __forceinline__ int piece_offset(int w) {
 // from call to call.
 template <int BITS, int MMAX>
 __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed, const uint16_t* __restrict__ cb,
-                                             const uint16_t* __restrict__ x, int64_t N, int64_t K, int M,
+                                             const uint16_t* x, int64_t N, int64_t K, int M,
                                              int64_t tile_id, int sa, int sb, bool wait_for_x, bool early_trigger,
                                              float& v) {
   using G = TGeo<BITS>;
@@ -107,7 +107,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
     for (int i = 0; i < NP; ++i) {
       v[i] = make_uint4(0, 0, 0, 0);
       if (px_k[i] >= 0 && (int64_t)s * G::kStepK + px_k[i] < K)
-        v[i] = __ldg(reinterpret_cast<const uint4*>(px_src[i] + (int64_t)s * G::kStepK));
+        v[i] = ld_input_u4(px_src[i] + (int64_t)s * G::kStepK);
     }
   };
 
@@ -275,7 +275,7 @@ __device__ __forceinline__ void store_output(float v, uint16_t* __restrict__ y, 
 template <int BITS, int MMAX>
 __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_cluster_kernel(const uint32_t* __restrict__ packed,
                                                                     const uint16_t* __restrict__ cb,
-                                                                    const uint16_t* __restrict__ x,
+                                                                    const uint16_t* x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, int early, int C) {
   __shared__ float shares[(kMaxCluster - 1) * kRows * 8];
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_cluster_kernel
 template <int BITS, int MMAX>
 __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_tiled_kernel(const uint32_t* __restrict__ packed,
                                                                     const uint16_t* __restrict__ cb,
-                                                                    const uint16_t* __restrict__ x,
+                                                                    const uint16_t* x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, int early) {
   const int steps = (int)((uint32_t)(K + TGeo<BITS>::kStepK - 1) / TGeo<BITS>::kStepK);
@@ -331,7 +331,7 @@ constexpr int kSlotFloats = kRows * 8 + 8;   // 128 sums (+ 8 unused: keeps the 
 template <int BITS, int MMAX>
 __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_split_kernel(const uint32_t* __restrict__ packed,
                                                                     const uint16_t* __restrict__ cb,
-                                                                    const uint16_t* __restrict__ x,
+                                                                    const uint16_t* x,
                                                                     uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                     int M, float* __restrict__ scratch) {
   const int64_t steps = tuned_row_steps(K, BITS);
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_split_kernel(c
 
 // Block c adds the two halves of the tile that the cut between CTA c and CTA c + 1 falls into.
 template <int BITS>
-__global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const float* __restrict__ scratch,
+__global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const float* scratch,
                                                                        const uint16_t* __restrict__ cb,
                                                                        uint16_t* __restrict__ y, int64_t N, int64_t K,
                                                                        int M, int ctas) {
@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const flo
   const int64_t row0 = (cut / steps) * kRows;
   const float* end_of_c = scratch + ((int64_t)blockIdx.x * 2 + 1) * kSlotFloats;
   const float* start_of_next = scratch + ((int64_t)(blockIdx.x + 1) * 2) * kSlotFloats;
-  const float v = end_of_c[threadIdx.x] + start_of_next[threadIdx.x];
+  const float v = __uint_as_float(ld_input_u32(end_of_c + threadIdx.x)) +
+                  __uint_as_float(ld_input_u32(start_of_next + threadIdx.x));
   store_output(v, y, N, M, row0);
 }
 

@@ -47,6 +47,25 @@ struct Indices {
   uint32_t sa, sb;   // block format: bf16 scales of rows g, g + 8
 };
 
+// Packed indices, scales and codebooks: constants of the layer for kmq_linear; the block format's interface does not say
+// so, there they may come from the previous kernel on the stream like the activations.
+template <bool BLOCK>
+__device__ __forceinline__ uint4 weights_u4(const void* p) {
+  return BLOCK ? ld_input_u4(p) : __ldg(static_cast<const uint4*>(p));
+}
+template <bool BLOCK>
+__device__ __forceinline__ uint2 weights_u2(const void* p) {
+  return BLOCK ? ld_input_u2(p) : __ldg(static_cast<const uint2*>(p));
+}
+template <bool BLOCK>
+__device__ __forceinline__ uint32_t weights_u32(const void* p) {
+  return BLOCK ? ld_input_u32(p) : __ldg(static_cast<const uint32_t*>(p));
+}
+template <bool BLOCK>
+__device__ __forceinline__ uint32_t weights_u16(const void* p) {
+  return BLOCK ? ld_input_u16(p) : __ldg(static_cast<const uint16_t*>(p));
+}
+
 // The lane's 16 indices of one row at `p`; of a canonical row's last group only what lies inside the row.
 template <int BITS, bool BLOCK>
 __device__ __forceinline__ void load_indices(const uint8_t* p, int left, uint32_t (&w)[RGeo<BITS, BLOCK>::kWords]) {
@@ -54,18 +73,18 @@ __device__ __forceinline__ void load_indices(const uint8_t* p, int left, uint32_
   for (int i = 0; i < RGeo<BITS, BLOCK>::kWords; ++i) w[i] = 0;
   if (left <= 0) return;
   if constexpr (BITS == 1) {
-    w[0] = __ldg(reinterpret_cast<const uint16_t*>(p));
+    w[0] = weights_u16<BLOCK>(p);
   } else if constexpr (BITS == 2) {
-    w[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+    w[0] = weights_u32<BLOCK>(p);
   } else if constexpr (BITS == 4 && BLOCK) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 v = weights_u2<BLOCK>(p);
     w[0] = v.x;
     w[1] = v.y;
   } else if constexpr (BITS == 4) {      // rows are whole words, no more
-    w[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
-    if (left > 8) w[1] = __ldg(reinterpret_cast<const uint32_t*>(p) + 1);
+    w[0] = weights_u32<BLOCK>(p);
+    if (left > 8) w[1] = weights_u32<BLOCK>(p + 4);
   } else {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint4 v = weights_u4<BLOCK>(p);
     w[0] = v.x;
     w[1] = v.y;
     w[2] = v.z;
@@ -89,11 +108,9 @@ __device__ __forceinline__ uint32_t weight_pair(const uint32_t (&w)[RGeo<BITS, B
 }
 
 template <int BITS, bool BLOCK, int NT, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_kernel(const uint8_t* __restrict__ wq,
-                                                                 const uint16_t* __restrict__ scales,
-                                                                 const uint16_t* __restrict__ cb,
-                                                                 const uint16_t* __restrict__ x,
-                                                                 uint16_t* __restrict__ y, int64_t N, int64_t K, int M) {
+__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_kernel(const uint8_t* wq,
+                                                                 const uint16_t* scales, const uint16_t* cb,
+                                                                 const uint16_t* x, uint16_t* y, int64_t N, int64_t K, int M) {
   using G = RGeo<BITS, BLOCK>;
   constexpr int AHEAD = Batch<NT>::kGroups;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -116,8 +133,8 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_ke
     load_indices<BITS, BLOCK>(pa + (int64_t)gi * 8 * BITS, left, q.wa);
     load_indices<BITS, BLOCK>(pb + (int64_t)gi * 8 * BITS, left, q.wb);
     if constexpr (BLOCK) {
-      q.sa = __ldg(scales + ra * groups + gi);
-      q.sb = __ldg(scales + rb * groups + gi);
+      q.sa = weights_u16<BLOCK>(scales + ra * groups + gi);
+      q.sb = weights_u16<BLOCK>(scales + rb * groups + gi);
     }
   };
   auto load_x = [&](int gi, uint32_t (&q)[NT][8]) {
@@ -127,8 +144,8 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_ke
       const int m = 8 * nt + g;
       const uint4* const src = reinterpret_cast<const uint4*>(px + (int64_t)m * K + (int64_t)gi * kGroup);
       uint4 v = make_uint4(0, 0, 0, 0), u = make_uint4(0, 0, 0, 0);
-      if (m < M && left > 0) v = __ldg(src);
-      if (m < M && left > 8) u = __ldg(src + 1);
+      if (m < M && left > 0) v = ld_input_u4(src);
+      if (m < M && left > 8) u = ld_input_u4(src + 1);
       q[nt][0] = v.x; q[nt][1] = v.y; q[nt][2] = v.z; q[nt][3] = v.w;
       q[nt][4] = u.x; q[nt][5] = u.y; q[nt][6] = u.z; q[nt][7] = u.w;
     }
@@ -148,8 +165,8 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 2 : 1) linear_rows_ke
   if constexpr (BLOCK) {
     for (int i = threadIdx.x; i < G::kEntries * 8; i += WARPS * 32) {   // four lanes' copies of an entry at a time
       const int e = i >> 3;
-      const uint32_t lo = __ldg(cb + (BITS == 8 ? e : e & ((1 << BITS) - 1)));
-      const uint32_t v = BITS == 8 ? lo : lo | ((uint32_t)__ldg(cb + (e >> BITS)) << 16);
+      const uint32_t lo = weights_u16<BLOCK>(cb + (BITS == 8 ? e : e & ((1 << BITS) - 1)));
+      const uint32_t v = BITS == 8 ? lo : lo | (weights_u16<BLOCK>(cb + (e >> BITS)) << 16);
       reinterpret_cast<uint4*>(table)[i] = make_uint4(v, v, v, v);
     }
   } else {
