@@ -35,6 +35,7 @@ def run_chain(layers, x0, M, sync):
     ws = torch.empty(max([l["ws_bytes"] for l in layers] + [16]), dtype=torch.uint8, device="cuda")
     outs, x = [], x0
     stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())      # the layers and x0 were made there
     with torch.cuda.stream(stream):
         for l in layers:
             y = torch.full((M * l["N"],), 0x7FC0, dtype=torch.int16, device="cuda")     # NaN patterns
