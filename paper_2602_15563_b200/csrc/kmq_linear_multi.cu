@@ -313,9 +313,9 @@ __global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* 
   // CTA c works on units [units c / ctas, units (c + 1) / ctas): unit u belongs to CTA ((u + 1) ctas - 1) / units
   const int64_t first = (int64_t)blockIdx.x * steps, last = first + steps - 1;
   const int64_t c0 = ((first + 1) * ctas - 1) / units, c1 = ((last + 1) * ctas - 1) / units;
-  if (c0 == c1) return;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // every block: this grid must not be complete before the first is
   asm volatile("griddepcontrol.launch_dependents;");
+  if (c0 == c1) return;
   const float4* const src = reinterpret_cast<const float4*>(scratch) + (int64_t)blockIdx.y * NT * 32 + threadIdx.x;
   constexpr int kSlot = TPC * NT * 32;
   float v[4];

@@ -354,7 +354,10 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_split_kernel(c
   asm volatile("griddepcontrol.launch_dependents;");
 }
 
-// Block c adds the two halves of the tile that the cut between CTA c and CTA c + 1 falls into.
+// Block c adds the two halves of the tile that the cut between CTA c and CTA c + 1 falls into.  Every block waits for the
+// first kernel, also one with nothing to add: where the tiles are a multiple of the CTAs no block has, and a grid whose
+// blocks all left at once would be complete before the first kernel is.  The next kernel on the stream waits for this grid
+// only and would read an unfinished y.
 template <int BITS>
 __global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const float* scratch,
                                                                        const uint16_t* __restrict__ cb,
@@ -363,9 +366,9 @@ __global__ void __launch_bounds__(kRows * 8) linear_split_fixup_kernel(const flo
   const int64_t steps = tuned_row_steps(K, BITS);
   const int64_t units = ((N + kRows - 1) / kRows) * steps;
   const int64_t cut = units * (blockIdx.x + 1) / ctas;
-  if (cut % steps == 0) return;   // the cut is a tile boundary: nothing was left partial
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the slots are the previous kernel's output
   asm volatile("griddepcontrol.launch_dependents;");
+  if (cut % steps == 0) return;   // the cut is a tile boundary: nothing was left partial
   const int64_t row0 = (cut / steps) * kRows;
   const float* end_of_c = scratch + ((int64_t)blockIdx.x * 2 + 1) * kSlotFloats;
   const float* start_of_next = scratch + ((int64_t)(blockIdx.x + 1) * 2) * kSlotFloats;
