@@ -16,8 +16,9 @@
  *     caller owns every buffer.  The library allocates no memory.  The state
  *     it keeps per device: a cache of device properties and of a few symbol
  *     addresses, two sticky error words in device memory (see
- *     kmq_device_error_flags) and the fixed 512 KiB scratch array of
- *     kmq_linear_static_scratch, which is part of the library image.
+ *     kmq_device_error_flags) and the fixed 640 KiB scratch array of
+ *     kmq_linear_static_scratch, which is part of the library image.  Per host
+ *     thread: the plans (kernel choices) of up to 64 shapes it used last.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).
  *     Work is enqueued on it and the call returns without synchronising,
  *     unless stated otherwise.
@@ -195,10 +196,12 @@ kmq_status kmq_linear_host(const uint32_t* packed, const uint16_t* codebooks, co
  * non-blocking callback), or a component that owns nothing but the buffers it
  * was given.  (This is a convenience of this library; the paper has no
  * counterpart.)  Same arguments, result and errors as kmq_linear.  Where
- * kmq_linear would need scratch (kmq_workspace_bytes() > 0) the partial sums
- * go to a fixed 512 KiB array that is part of the library image on every GPU
- * that loads it (kmq_static_scratch_capacity() returns the size); a shape that
- * needs more is refused with KMQ_ERR_SCRATCH_LIMIT and nothing is launched.
+ * kmq_linear would use scratch (kmq_workspace_bytes() > 0) the partial sums
+ * go to a fixed 640 KiB array that is part of the library image on every GPU
+ * that loads it (kmq_static_scratch_capacity() returns the size).  A shape that
+ * uses more runs as kmq_linear runs it without a workspace where that is
+ * possible ("multi_balanced_*": another order of the sum, slower) and is
+ * otherwise refused with KMQ_ERR_SCRATCH_LIMIT and nothing is launched.
  * The call never allocates or frees memory.
  *   - The first call on each device looks up the array's device address
  *     (once, with that device current); make that first call outside any

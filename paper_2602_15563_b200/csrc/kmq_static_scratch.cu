@@ -1,7 +1,7 @@
 // kmq_linear_static_scratch: kmq_linear for callers that cannot hand over a scratch buffer.
 //
-// Some shapes of kmq_linear (long rows, more 16-row tiles than the GPU keeps resident) run the balanced kernel pair,
-// which parks partial sums in global scratch memory between its two launches.  kmq_linear takes that scratch from the
+// Some shapes of kmq_linear (more 16-row tiles than the GPU keeps resident, or a last wave that leaves it half empty) run
+// a balanced kernel pair, which parks partial sums in global scratch memory between its two launches.  kmq_linear takes that scratch from the
 // caller, who normally gets it from cudaMalloc or a framework allocator.  A caller that must not allocate -- code
 // running inside a region where the allocator is locked or allocation is forbidden (a real-time control loop, a
 // callback that may not block, a plug-in that was handed only its input and output buffers, a process whose memory
@@ -14,8 +14,9 @@
 namespace {
 
 // The scratch itself: part of the library's device image, present on every GPU that loads the library until the
-// process exits.  512 KiB covers the balanced kernel pair on GPUs with up to 160 SMs (3 * SMs * 1088 bytes).
-constexpr size_t kStaticScratchBytes = 512u * 1024u;
+// process exits.  On GPUs with up to 160 SMs 640 KiB cover the balanced pair of one or two batch rows (3 * 1088 bytes per
+// SM) and the balanced form of the multi-tile kernel with 8 tiles per SM and up to 8 rows (4096 bytes per SM).
+constexpr size_t kStaticScratchBytes = 640u * 1024u;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 // In host code `g_static_scratch` is only a handle for the runtime, not an address a kernel may use; the device
@@ -48,8 +49,8 @@ extern "C" kmq_status kmq_linear_static_scratch(const uint32_t* packed, const ui
                                                 void* stream) {
   // 0 both for shapes that need no scratch and for invalid arguments: kmq_linear sorts those out
   size_t need = kmq_workspace_bytes(N, K, bits, M, layout);
-  // only what cannot run without: the array is shared by all streams
-  if (need > 0) need = kmq::plan_linear(N, K, bits, M, layout, 0).workspace;
+  // a plan that only gains by scratch, not needs it, gives way to the one without where the array is too small
+  if (need > kStaticScratchBytes) need = kmq::plan_linear(N, K, bits, M, layout, kStaticScratchBytes).workspace;
   if (need == 0) return kmq_linear(packed, codebooks, x, y, N, K, bits, M, layout, nullptr, 0, stream);
   if (need > kStaticScratchBytes) return KMQ_ERR_SCRATCH_LIMIT;
   cudaError_t err = cudaSuccess;

@@ -53,3 +53,27 @@ def test_static_scratch_passes_through_shapes_without_scratch_and_bad_arguments(
     assert torch.equal(y1, y2)
     assert kmq.kmq_linear_static_scratch(packed, cb, x, y2, N, K, 3, M, check=False) == kmq.KMQ_ERR_BITS
     assert kmq.kmq_linear_static_scratch(0, cb, x, y2, N, K, bits, M, check=False) == kmq.KMQ_ERR_NULL
+
+
+@pytest.mark.parametrize("N,K,bits,M", [(10240, 8192, 4, 4), (10230, 16384, 2, 8), (8192, 28672, 4, 16)])
+def test_balanced_form_of_the_multi_tile_kernel(N, K, bits, M):
+    """Same kernels, so the same bits, as kmq_linear with a workspace where the array is large enough for the partial sums;
+    as kmq_linear without one where it is not (the last shape)."""
+    T = kmq.KMQ_LAYOUT_TUNED
+    need = kmq.kmq_workspace_bytes(N, K, bits, M, T)
+    assert need > 0 and kmq.kmq_linear_variant(N, K, bits, M, T).startswith("multi_balanced")
+    fits = need <= kmq.kmq_static_scratch_capacity()
+    assert fits == (M <= 8)
+    g = torch.Generator(device="cuda").manual_seed(N + M)
+    words = kmq.kmq_packed_bytes(N, K, bits, T) // 4
+    packed = torch.randint(-2**31, 2**31 - 1, (words,), dtype=torch.int32, device="cuda", generator=g)
+    cb = (torch.randn(N, 1 << bits, device="cuda", generator=g) * 0.02).sort(dim=1).values.to(torch.bfloat16)
+    x = torch.randn(M, K, device="cuda", generator=g).to(torch.bfloat16)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    y, with_ws, without = (torch.zeros(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(3))
+    kmq.kmq_linear(packed, cb, x, with_ws, N, K, bits, M, ws, need, layout=T)
+    kmq.kmq_linear(packed, cb, x, without, N, K, bits, M, None, 0, layout=T)
+    kmq.kmq_linear_static_scratch(packed, cb, x, y, N, K, bits, M, layout=T)
+    torch.cuda.synchronize()
+    assert not torch.equal(with_ws, without)             # the two forms can be told apart
+    assert torch.equal(y, with_ws if fits else without)
