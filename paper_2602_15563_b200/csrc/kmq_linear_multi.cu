@@ -313,8 +313,13 @@ __global__ void __launch_bounds__(32 * NT) linear_multi_sum_kernel(const float* 
   // CTA c works on units [units c / ctas, units (c + 1) / ctas): unit u belongs to CTA ((u + 1) ctas - 1) / units
   const int64_t first = (int64_t)blockIdx.x * steps, last = first + steps - 1;
   const int64_t c0 = ((first + 1) * ctas - 1) / units, c1 = ((last + 1) * ctas - 1) / units;
+  // At b = 4 the next call's CTAs set up (tables) under the first kernel's MMAs, as they do without this kernel: it releases
+  // them before its own wait (8192 x 28672, M = 3 45.6 -> 44.9 us; 8192 x 16384 29.1 -> 28.6).  With more than 8 batch rows
+  // and at b = 1, 2, where the set-up is short, that gave nothing or cost up to 1 %.
+  constexpr bool kEarly = BITS == 4 && NT == 1;
+  if constexpr (kEarly) asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");   // every block: this grid must not be complete before the first is
-  asm volatile("griddepcontrol.launch_dependents;");
+  if constexpr (!kEarly) asm volatile("griddepcontrol.launch_dependents;");
   if (c0 == c1) return;
   const float4* const src = reinterpret_cast<const float4*>(scratch) + (int64_t)blockIdx.y * NT * 32 + threadIdx.x;
   constexpr int kSlot = TPC * NT * 32;
@@ -499,23 +504,33 @@ static cudaError_t launch_multi(int bits, const MultiCall& c) {
 }
 
 // Whether the balanced form is used (ctas > 0), and its scratch.  It saves the steps in which the last wave leaves CTA
-// slots empty and costs about 9000 clocks: the second kernel, and a CTA's start on one or two more groups.  An SM does
-// some 20 weights per clock (24 at b = 2), 27 up to 8 batch rows, 12 with more than 16.  us per call, without / with:
-// 8192 x 28672, M = 16 (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4,
-// M = 16 32.5 / 25.6, b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 12288 x 4096, b = 2, M = 12
-// 12.9 / 13.5.
+// slots empty and costs the second kernel and a CTA's start on one or two more groups.  us per call, without / with:
+//   up to 8 batch rows, from sweeps of 76 to 650 groups by 8 to 192 steps at M = 8 (3 and 8 at b = 4): the cost is that of
+//          172 thousand weights on an SM, whose share the saved steps have to exceed (b = 1: 12288 x 4096, 164, 9.8 / 10.3,
+//          16384 x 12288, 213, 27.1 / 26.0; b = 2: 8192 x 16384, 142, 19.4 / 19.5, 5120 x 8192, 241, 10.9 / 9.5).  At b = 2
+//          in two waves or more 384: the CTAs of a last wave have an SM to themselves and finish early (12288 x 4096, 184,
+//          10.8 / 11.7, 9600 x 6144, 387, 13.3 / 12.5).  At b = 4 165 (5632 x 6144, 159, 12.0 / 12.2, 6400 x 8192, 170,
+//          15.5 / 15.2), 140 where the groups nearly fill the SMs, so that few are shared by more than two CTAs
+//          (8192 x 16384, 142, M = 3 28.4 / 28.6, M = 8 29.5 / 29.4; 8192 x 20480, 177, 36.0 / 35.0).
+//   more   some 9000 clocks, of which an SM does 20 weights each (24 at b = 2), 12 with more than 16 rows.  8192 x 28672,
+//          M = 16 (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4,
+//          M = 16 32.5 / 25.6, b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 12288 x 4096, b = 2,
+//          M = 12 12.9 / 13.5.
 MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
   MultiSplit sp = {};
   const DeviceInfo* di = device_info();
   if (!di || M > linear_multi_rows_per_launch(bits)) return sp;
   if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess) return {};
-  const int64_t steps = tuned_row_steps(K, bits);
+  const int64_t steps = tuned_row_steps(K, bits), sms = di->sm_count;
   // CTAs that have an SM to themselves run as fast as the SM lets them: then it is the SMs that are empty, not the slots
-  const int64_t slots = sp.groups <= di->sm_count ? di->sm_count : sp.ctas, waves = (sp.groups + slots - 1) / slots;
+  const int64_t slots = sp.groups <= sms ? sms : sp.ctas, waves = (sp.groups + slots - 1) / slots;
   const double saved = (double)(waves * slots - sp.groups) / slots * (double)steps;
-  const double step_clocks =
-      (double)(slots / di->sm_count) * sp.tiles * (kTileRows * 512 / bits) / (M > 16 ? 12.0 : M <= 8 ? 27.0 : bits == 2 ? 24.0 : 20.0);
-  return saved * step_clocks > 9000.0 && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
+  const double weights = saved * (double)(slots / sms) * sp.tiles * (kTileRows * 512 / bits);   // of one SM
+  double cost;
+  if (M > 8) cost = 9000.0 * (M > 16 ? 12.0 : bits == 2 ? 24.0 : 20.0);
+  else if (bits == 4) cost = sp.groups <= sms && 6 * sp.groups >= 5 * sms ? 140e3 : 165e3;
+  else cost = bits == 2 && waves > 1 ? 384e3 : 172e3;
+  return weights > cost && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
 }
 
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
