@@ -471,30 +471,45 @@ cudaError_t launch_bits(const MultiCall& c) {
 int linear_multi_rows_per_launch(int bits) { return bits == 1 ? 32 : 64; }
 
 // Smallest batch that goes to the multi-tile kernel.  The GEMV kernel stages the activations once per tile, here the tiles
-// of a CTA share them; but its grid is finer, and it shares K among a cluster.  us per call, GEMV / multi-tile:
-//   b = 1  more than three tiles per SM: 2 rows on.  Otherwise up to 4 rows stay (1024 x 8192, M = 3 3.5 / 5.4; 6144 x 8192,
-//          M = 4 8.4 / 9.8) except on long rows (2048 x 28672, M = 3 11.2 / 10.6) and on few steps that two CTAs of one SM
-//          and one of another share badly (3072 x 3072, M = 3 3.6 / 3.4).
-//   b = 2  waves: 5 rows on, on long rows 2 (8192 x 28672, M = 2 34.0 / 30.0).  One wave: 9, on long rows 2 where the
-//          GEMV kernel does not use clusters (4096 x 9216, M = 2 9.2 / 7.1, M = 8 11.8 / 8.1), 5 where it uses two CTAs on
-//          a full machine (3072 x 16384, M = 4 9.6 / 10.4, M = 8 11.5 / 10.9).
-//   b = 4  from 3 rows on the GEMV kernel's tables leave room for two CTAs per SM: 3 where the tiles do not fit these slots
-//          (6144 x 4096, M = 3 9.1 / 8.3, M = 8 11.1 / 8.7) and on long rows (3072 x 16384, M = 4 16.2 / 15.0); 7 on
-//          medium ones (4096 x 4096, M = 8 6.3 / 5.6; 3072 x 8192 9.9 / 8.8); else 9.
+// of a CTA share them; but its grid is finer, and it shares K among a cluster.  The lines below are from a sweep of 20 to
+// 1024 tiles by 4 to 224 steps at every batch up to 8, both kernels on all of it; us per call, GEMV / multi-tile:
+//   More than three tiles per SM.  The multi-tile kernel has the better of it up to four, where its groups are one wave;
+//   with up to six the second wave is nearly empty, and on short rows the finer grid wins.
+//     b = 1  2 rows on (8192 x 4096, M = 2 5.6 / 6.0, M = 3 6.3 / 6.0).  Beyond four tiles per SM 3 with 4 to 32 steps, of
+//            more than six tiles 8 to 32 (9600 x 4096, M = 2 6.3 / 9.2), and 5 with 4 to 12 steps of up to five tiles
+//            (11008 x 4096, M = 3 7.6 / 9.6).  Not on shorter rows (9600 x 1024, M = 2 and 3 13 and 25 % faster here).
+//     b = 2  5 rows on (8192 x 4096, M = 5 7.7 / 6.6; M = 4 6.8 / 6.6, but 9600 x 4096, M = 4 7.8 / 9.2), on long rows 2
+//            (7200 x 24576, M = 2 28.6 / 24.1).
+//     b = 4  from two tiles per SM on, where the GEMV kernel's tables leave room for two CTAs per SM from 3 rows on: 3
+//            (8192 x 4096, M = 3 9.4 / 8.4), 5 with 13 to 32 steps of four to six tiles (12288 x 4096, M = 3 13.7 / 15.2;
+//            11008 x 2048, M = 3 7.5 / 8.6; 11008 x 8192 23.6 / 21.9).
+//   Fewer tiles.
+//     b = 1  5 (1024 x 8192, M = 3 3.5 / 5.4; 6144 x 8192, M = 4 8.4 / 9.8), on long rows 3 (4160 x 24576, M = 3
+//            15.1 / 14.1), and with an even number of steps below 8 on one to one and a half tiles per SM (3072 x 3072,
+//            M = 3 3.6 / 3.4; an odd number is slower by 2 to 11 % on nine widths, 3072 x 2560 3.1 / 3.4).
+//     b = 2  9.  On long rows 2 with one and a half to two tiles per SM (4160 x 10240, M = 3 9.8 / 7.9); 5 below that, where
+//            the GEMV kernel uses clusters (2976 x 16384, M = 4 9.6 / 10.5, M = 8 11.5 / 11.0), with less than a tile per SM
+//            from 64 steps on (1600 x 16384, M = 8 9.4 / 8.6, but 2336 x 10240, M = 4 5.4 / 7.7) and 2 from 81 on
+//            (1600 x 24576, M = 4 10.9 / 9.7).
+//     b = 4  9.  With one to two tiles per SM 3 on long rows (2976 x 16384, M = 3 15.4 / 14.3) and 7 on medium ones
+//            (4160 x 8192, M = 8 10.5 / 9.0).
 int linear_multi_min_rows(int bits, int64_t N, int64_t K) {
   const DeviceInfo* di = device_info();
   const int64_t sms = di ? di->sm_count : 148, tiles = (N + kTileRows - 1) / kTileRows, steps = tuned_row_steps(K, bits);
-  const bool waves = tiles > sms * 3;
+  const bool second_wave = tiles > 4 * sms && tiles <= 6 * sms;
   if (bits == 1) {
-    if (waves) return 2;
-    return steps > 32 || (steps < 8 && tiles > sms && 2 * tiles <= 3 * sms) ? 3 : 5;
+    if (tiles > 4 * sms && steps >= (second_wave ? 4 : 8) && steps <= 32) return steps <= 12 && tiles <= 5 * sms ? 5 : 3;
+    if (tiles > 3 * sms) return 2;
+    return steps > 32 || (steps < 8 && steps % 2 == 0 && tiles > sms && 2 * tiles <= 3 * sms) ? 3 : 5;
   }
   if (bits == 2) {
-    if (waves) return steps > 64 ? 2 : 5;
+    if (tiles > 3 * sms) return steps > 64 ? 2 : 5;
     if (steps <= 32 || 2 * tiles <= sms || tiles > 2 * sms) return 9;
-    return tiles > sms && 2 * tiles <= 3 * sms ? 5 : 2;
+    if (2 * tiles > 3 * sms) return 2;
+    if (tiles > sms) return 5;
+    return steps > 80 ? 2 : steps >= 64 ? 5 : 9;
   }
-  if (tiles > 2 * sms) return 3;
+  if (tiles > 2 * sms) return second_wave && steps > 12 && steps <= 32 ? 5 : 3;
   if (tiles <= sms || steps < 32) return 9;
   return steps > 64 ? 3 : 7;
 }
@@ -505,13 +520,14 @@ static cudaError_t launch_multi(int bits, const MultiCall& c) {
 
 // Whether the balanced form is used (ctas > 0), and its scratch.  It saves the steps in which the last wave leaves CTA
 // slots empty and costs the second kernel and a CTA's start on one or two more groups.  us per call, without / with:
-//   up to 8 batch rows, from sweeps of 76 to 650 groups by 8 to 192 steps at M = 8 (3 and 8 at b = 4): the cost is that of
-//          172 thousand weights on an SM, whose share the saved steps have to exceed (b = 1: 12288 x 4096, 164, 9.8 / 10.3,
-//          16384 x 12288, 213, 27.1 / 26.0; b = 2: 8192 x 16384, 142, 19.4 / 19.5, 5120 x 8192, 241, 10.9 / 9.5).  At b = 2
-//          in two waves or more 384: the CTAs of a last wave have an SM to themselves and finish early (12288 x 4096, 184,
-//          10.8 / 11.7, 9600 x 6144, 387, 13.3 / 12.5).  At b = 4 165 (5632 x 6144, 159, 12.0 / 12.2, 6400 x 8192, 170,
-//          15.5 / 15.2), 140 where the groups nearly fill the SMs, so that few are shared by more than two CTAs
-//          (8192 x 16384, 142, M = 3 28.4 / 28.6, M = 8 29.5 / 29.4; 8192 x 20480, 177, 36.0 / 35.0).
+//   up to 8 batch rows, from sweeps of 20 to 1300 groups by 8 to 224 steps: the cost, in thousands of weights on an SM, which
+//          the weights of the steps saved have to exceed, is 190 at b = 1 (12288 x 4096, 184, M = 3 9.8 / 10.3;
+//          16384 x 12288, 213, M = 8 27.1 / 26.0), 172 at b = 2 (8192 x 16384, 142, M = 3 19.4 / 19.5; 5120 x 8192, 241,
+//          M = 8 10.9 / 9.5), but 340 there in two waves or more: the CTAs of a last wave have an SM to themselves and finish
+//          early (12288 x 4096, 184, M = 8 10.8 / 11.7; 9600 x 6144, 387, 13.3 / 12.5).  At b = 4 165 (5632 x 6144, 159,
+//          M = 8 12.0 / 12.2; 6400 x 8192, 170, 15.5 / 15.3), 140 where the groups nearly fill the SMs, so that few are
+//          shared by more than two CTAs (8192 x 16384, 142, M = 3 28.4 / 28.6, M = 8 29.5 / 29.4; 8192 x 20480, 177,
+//          M = 8 36.0 / 35.0).
 //   more   some 9000 clocks, of which an SM does 20 weights each (24 at b = 2), 12 with more than 16 rows.  8192 x 28672,
 //          M = 16 (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4,
 //          M = 16 32.5 / 25.6, b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 12288 x 4096, b = 2,
@@ -529,7 +545,7 @@ MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
   double cost;
   if (M > 8) cost = 9000.0 * (M > 16 ? 12.0 : bits == 2 ? 24.0 : 20.0);
   else if (bits == 4) cost = sp.groups <= sms && 6 * sp.groups >= 5 * sms ? 140e3 : 165e3;
-  else cost = bits == 2 && waves > 1 ? 384e3 : 172e3;
+  else cost = bits == 1 ? 190e3 : waves > 1 ? 340e3 : 172e3;
   return weights > cost && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
 }
 
