@@ -32,9 +32,18 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _torch_include() -> str:
-    """torch's header folder (the extension module uses its DLPack header), found without importing torch."""
-    return os.path.join(os.path.dirname(importlib.util.find_spec("torch").origin), "include")
+def _torch_include() -> list[str]:
+    """torch's header folder as an include option (the extension module uses its DLPack header where it has the exchange
+    table), found without importing torch; nothing where torch is not installed."""
+    spec = importlib.util.find_spec("torch")
+    return ["-I", os.path.join(os.path.dirname(spec.origin), "include")] if spec and spec.origin else []
+
+
+def native_command(out: str, torch_include: list[str]) -> list[str]:
+    """How the extension module is compiled and linked: host code only; it finds libkmq.so beside itself at run time."""
+    return [_nvcc(), "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I",
+            sysconfig.get_paths()["include"], *torch_include, NATIVE_SRC, "-L", PKG_DIR, "-l:libkmq.so", "-Xlinker",
+            "-rpath=$ORIGIN", "-o", out]
 
 
 def needs_build() -> bool:
@@ -78,11 +87,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed linking libkmq.so")
     os.replace(LIB_PATH + ".tmp", LIB_PATH)
 
-    # host code only; finds libkmq.so beside itself at run time
-    res = subprocess.run([_nvcc(), "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I",
-                          os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", _torch_include(), NATIVE_SRC,
-                          "-L", PKG_DIR, "-l:libkmq.so", "-Xlinker", "-rpath=$ORIGIN", "-o", NATIVE_PATH + ".tmp"],
-                         capture_output=True, text=True)
+    res = subprocess.run(native_command(NATIVE_PATH + ".tmp", _torch_include()), capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("building the extension module failed")

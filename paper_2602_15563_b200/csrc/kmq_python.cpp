@@ -7,11 +7,21 @@
 // layer for the tensors and the stream.  The GIL is released around the library call, as ctypes does.
 //
 // torch tensors go through torch's DLPack exchange table (a C function per tensor, and one for the current stream); what
-// it does not describe, or another tensor library's object, is asked for data_ptr() instead.
+// it does not describe, or another tensor library's object, is asked for data_ptr() instead.  Built against a torch whose
+// headers do not have the table (it came with DLPack 1.3; 2.11 has it), everything is.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#if defined(__has_include)
+#if __has_include(<ATen/dlpack.h>)
 #include <ATen/dlpack.h>
+#endif
+#endif
+#if defined(DLPACK_MAJOR_VERSION) && defined(DLPACK_MINOR_VERSION)
+#if DLPACK_MAJOR_VERSION > 1 || (DLPACK_MAJOR_VERSION == 1 && DLPACK_MINOR_VERSION >= 3)
+#define KMQ_HAVE_EXCHANGE_TABLE 1
+#endif
+#endif
 
 #include <stdint.h>
 #include <string.h>
@@ -31,9 +41,11 @@ PyObject* s_cuda_stream;
 PyObject* s_numel;
 PyObject* s_element_size;
 PyObject* g_error = nullptr;          // KmqError, handed over by the Python module
+#ifdef KMQ_HAVE_EXCHANGE_TABLE
 PyTypeObject* g_tensor_type = nullptr;               // torch.Tensor, once one was seen
 const DLPackExchangeAPI* g_exchange = nullptr;       // its exchange table
 bool g_cuda_ready = false;                           // torch's CUDA side is set up
+#endif
 
 // ---- one argument -> one C value; false with a Python error set ----
 bool to_c(PyObject* o, int64_t* v) {
@@ -49,6 +61,7 @@ bool to_c(PyObject* o, size_t* v) {
   *v = PyLong_AsSize_t(o);
   return !(*v == (size_t)-1 && PyErr_Occurred());
 }
+#ifdef KMQ_HAVE_EXCHANGE_TABLE
 // Finds torch's exchange table; called with an object whose type may be torch.Tensor.
 void find_exchange(PyObject* o) {
   PyTypeObject* const type = Py_TYPE(o);
@@ -66,6 +79,7 @@ void find_exchange(PyObject* o) {
   Py_XDECREF(capsule);
   PyErr_Clear();
 }
+#endif
 
 // None, an address, or an object with data_ptr()
 bool to_address(PyObject* o, void** v) {
@@ -77,6 +91,7 @@ bool to_address(PyObject* o, void** v) {
     *v = PyLong_AsVoidPtr(o);
     return *v || !PyErr_Occurred();
   }
+#ifdef KMQ_HAVE_EXCHANGE_TABLE
   if (!g_tensor_type) find_exchange(o);
   if (Py_TYPE(o) == g_tensor_type) {
     DLTensor t;
@@ -86,6 +101,7 @@ bool to_address(PyObject* o, void** v) {
     }
     PyErr_Clear();   // e.g. a type that DLPack has no name for
   }
+#endif
   PyObject* r = PyObject_CallMethodNoArgs(o, s_data_ptr);
   if (!r) return false;
   *v = PyLong_AsVoidPtr(r);
@@ -103,17 +119,21 @@ bool to_c(PyObject* o, T** v) {
 // torch's current stream on the current device.  The first call goes through torch's public object, which also sets
 // CUDA up.
 bool current_stream(void** stream) {
+#ifdef KMQ_HAVE_EXCHANGE_TABLE
   if (g_cuda_ready && g_exchange) {
     const int dev = kmq_internal_current_device();
     if (dev >= 0) return g_exchange->current_work_stream(kDLCUDA, dev, stream) == 0;
   }
+#endif
   PyObject* cuda = PyImport_ImportModule("torch.cuda");
   PyObject* st = cuda ? PyObject_CallMethod(cuda, "current_stream", nullptr) : nullptr;
   PyObject* r = st ? PyObject_GetAttr(st, s_cuda_stream) : nullptr;
   Py_XDECREF(cuda);
   Py_XDECREF(st);
   if (!r) return false;
+#ifdef KMQ_HAVE_EXCHANGE_TABLE
   g_cuda_ready = true;
+#endif
   *stream = PyLong_AsVoidPtr(r);
   Py_DECREF(r);
   return *stream || !PyErr_Occurred();
