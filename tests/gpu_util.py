@@ -154,3 +154,42 @@ def block_table_from_bytes(wq: np.ndarray, scales: np.ndarray, K: int, bits: int
     mask = scb != 0
     out[mask] = scb[mask]
     return out
+
+
+def launched_kernels(enqueue):
+    """What `enqueue()` launches, without running it: it is captured on a stream of its own, and the kernel nodes of the
+    graph are read back in order as (function name, grid, block, CTAs per cluster)."""
+    from cuda.bindings import driver as cu
+
+    def ok(res):
+        assert res[0] == cu.CUresult.CUDA_SUCCESS, res[0]
+        return res[1] if len(res) == 2 else res[1:]
+
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        enqueue()
+    raw = cu.CUgraph(graph.raw_cuda_graph())
+    count = ok(cu.cuGraphGetNodes(raw, 0))[1]
+    nodes = ok(cu.cuGraphGetNodes(raw, count))[0]
+    out = []
+    for node in nodes[:count]:
+        if ok(cu.cuGraphNodeGetType(node)) != cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        p = ok(cu.cuGraphKernelNodeGetParams(node))
+        name = ok(cu.cuFuncGetName(p.func)) if int(p.func) else ok(cu.cuKernelGetName(p.kern))
+        cluster = ok(cu.cuGraphKernelNodeGetAttribute(node, cu.CUkernelNodeAttrID.CU_LAUNCH_ATTRIBUTE_CLUSTER_DIMENSION))
+        dim = cluster.clusterDim                                  # all 0 without clusters
+        out.append((name.decode(), (p.gridDimX, p.gridDimY, p.gridDimZ), p.blockDimX, max(1, dim.x * dim.y * dim.z)))
+    return out
+
+
+def linear_kernels(N, K, bits, M, layout, workspace=True):
+    """launched_kernels of a kmq_linear call of that shape."""
+    packed = torch.zeros(kmq.kmq_packed_bytes(N, K, bits, layout), dtype=torch.uint8, device="cuda")
+    cb = torch.zeros(N << bits, dtype=torch.int16, device="cuda")
+    x, y = (torch.zeros(M * n, dtype=torch.int16, device="cuda") for n in (K, N))
+    nbytes = kmq.kmq_workspace_bytes(N, K, bits, M, layout) if workspace else 0
+    ws = torch.empty(max(nbytes, 16), dtype=torch.uint8, device="cuda")
+    return launched_kernels(lambda: kmq.kmq_linear(packed, cb, x, y, N, K, bits, M, ws, nbytes, layout=layout))

@@ -1,0 +1,81 @@
+"""Which kernel, in which form, the shapes of the parity tests reach (148 SMs): the parity tests compare results, which would
+not change if another kernel ran.  The launches are read from a captured graph."""
+import re
+
+import numpy as np
+import pytest
+
+from oracle import kmq_oracle as orc
+from paper_2602_15563_b200 import kmq
+from tests import gpu_util as gu
+from tests.test_gpu_tcgen05 import random_layer, run
+
+pytestmark = pytest.mark.gpu
+TUNED, CANONICAL = kmq.KMQ_LAYOUT_TUNED, kmq.KMQ_LAYOUT_CANONICAL
+
+
+def template(name, kernel):
+    """Template arguments of a mangled kernel name, or None for another kernel."""
+    m = re.search(rf"\d{kernel}I((?:L[ib]\d+E)+)E", name)
+    return tuple(int(v) for v in re.findall(r"L[ib](\d+)E", m.group(1))) if m else None
+
+
+@pytest.mark.parametrize("bits", (1, 2, 4))
+@pytest.mark.parametrize("N,K,M,size", [(1, 28672, 1, 8), (100, 20000, 2, 8), (250, 28640, 1, 8), (500, 16416, 1, 4),
+                                        (590, 16352, 4, 4), (1030, 12288, 1, 2), (3070, 8224, 1, 2), (700, 20000, 8, 2)])
+def test_clusters_of_the_gemv_kernel(bits, N, K, M, size):
+    if bits == 1 and (N, M) in ((3070, 1), (700, 8)):    # b = 1: a step takes the SM longer; 5 rows and more go elsewhere
+        size = 1 if M == 1 else None
+    (name, grid, _, cluster), *rest = gu.linear_kernels(N, K, bits, M, TUNED)
+    if size is None:
+        assert template(name, "linear_multi_kernel")
+        return
+    kernel = "linear_cluster_kernel" if size > 1 else "linear_tiled_kernel"
+    assert not rest and template(name, kernel) == (bits, M)
+    assert cluster == size and grid == (-(-N // 16) * size, 1, 1)
+
+
+@pytest.mark.parametrize("N,K,M,form", [
+    (17, 136, 9, (2, 2, 8)), (100, 4160, 16, (2, 2, 16)), (5000, 392, 16, (2, 4, 16)), (20000, 520, 16, (2, 2, 8)),
+    (9480, 1536, 3, (1, 2, 8)), (4160, 4096, 7, (1, 2, 16)), (8190, 264, 4, (1, 4, 16)),
+])
+def test_every_shape_of_cta_of_the_half_tables(N, K, M, form):
+    (name, _, threads, _), = gu.linear_kernels(N, K, 4, M, TUNED)
+    assert template(name, "linear_multi_kernel") == (4, *form, 0) and threads == 32 * form[2]
+
+
+@pytest.mark.parametrize("bits,N,K,M", [(4, 10230, 8192, 16), (4, 8200, 28672, 9), (2, 10240, 8192, 32), (1, 9500, 20000, 9),
+                                        (4, 2050, 28680, 12), (2, 5130, 16400, 40), (4, 7365, 16544, 3)])
+def test_balanced_form_is_two_kernels(bits, N, K, M):
+    main, add = gu.linear_kernels(N, K, bits, M, TUNED)
+    form = template(main[0], "linear_multi_kernel")
+    assert form[0] == bits and form[4] == 1 and main[1][0] % 148 == 0
+    assert template(add[0], "linear_multi_sum_kernel") == form[:3]
+    plain, = gu.linear_kernels(N, K, bits, M, TUNED, workspace=False)
+    assert template(plain[0], "linear_multi_kernel") == (*form[:4], 0)
+
+
+@pytest.mark.parametrize("N,K,M", [(256, 512, 129), (16, 64, 300), (129, 640, 161), (1000, 1024, 520), (5000, 256, 1100)])
+def test_prefill_runs_on_cta_pairs(N, K, M):
+    (name, grid, _, cluster), = gu.linear_kernels(N, K, 2, M, TUNED)
+    assert template(name, "linear_umma_pair_kernel") == (2,) and cluster == 2 and grid[0] % 2 == 0
+
+
+@pytest.mark.parametrize("bits,N,K,M,ksplit", [(2, 2100, 4096, 200, 2), (2, 4800, 4096, 256, 1), (1, 257, 4224, 256, 2),
+                                               (4, 300, 4096, 150, 2)])
+def test_single_cta_kernel_with_several_batch_tiles(bits, N, K, M, ksplit):
+    (name, grid, _, cluster), = gu.linear_kernels(N, K, bits, M, TUNED)
+    assert template(name, "linear_umma_kernel") == (bits, 128)
+    assert grid == (-(-N // 128), ksplit, -(-M // 128)) and cluster == ksplit
+    rng = np.random.default_rng(N + M)
+    idx, cb, x = random_layer(rng, N, K, bits, M)
+    y_ref, s = orc.linear_f64(orc.pack_canonical(idx, bits), cb, x, K, bits)
+    assert orc.check_linear(run(idx, cb, x, bits), y_ref, s) <= 1.0
+
+
+@pytest.mark.parametrize("bits", (1, 2, 4))
+@pytest.mark.parametrize("N,words,M,warps", [(17, 5, 9, 16), (2400, 41, 3, 8)])
+def test_canonical_rows(bits, N, words, M, warps):
+    kernels = gu.linear_kernels(N, words * (32 // bits), bits, M, CANONICAL)
+    assert len(kernels) == -(-M // 8)
+    assert all(template(k[0], "linear_rows_kernel") == (bits, 0, 1, warps) for k in kernels)
