@@ -335,8 +335,12 @@ kmq_status kmq_block_dequant_to_bf16(const uint8_t* wq, const uint16_t* scales, 
  * kmq_block_table_linear -- y[m, n] = sum_k x[m, k] * scale[n, k/64] *
  *   c[idx[n, k]]: fp32 tables, fp32 accumulation, bf16 result, the tolerance
  *   stated for kmq_linear for any finite codebook (a table entry is the sum of
- *   the selected products themselves).  One pass over the weights per batch
- *   row: meant for M = 1 .. 4.  Two launches per pass when scratch is needed.
+ *   the selected products themselves).  `table` and `codebook` are treated as
+ *   constants of the layer, as packed and codebooks of kmq_linear: they may be
+ *   read before earlier work on `stream` has finished, and must not be written
+ *   by a foreign kernel that signals an early launch of its dependents.
+ *   (kmq_block_linear reads nothing before earlier work has finished.)  One
+ *   pass over the weights per batch row: meant for M = 1 .. 4.  Two launches per pass when scratch is needed.
  *   Waits on copies are bounded; a run-out is reported by
  *   kmq_device_error_flags only.  Needs 227 KB of shared memory per CTA
  *   (KMQ_ERR_CUDA otherwise).
@@ -377,7 +381,7 @@ kmq_status kmq_block_table_linear(const uint8_t* table, const uint16_t* codebook
  *   bits       1, 2, 4 or 8 (8 for the shared codebook of the block format).
  *   codebooks  DEVICE bf16 [N, 2^bits], non-decreasing along a row.
  *   centroids  DEVICE float64 [N, 2^bits] or NULL: the unrounded centroids.
- *   A row is sorted in shared memory: 2^bits <= K <= 32768, else KMQ_ERR_SHAPE.
+ *   A row is held in shared memory: 2^bits <= K <= 32768, else KMQ_ERR_SHAPE.
  * kmq_assign_pack -- packed[n, k] = index of the centroid of codebooks[n, :]
  *   nearest to W[n, k], written directly in `layout` (the argument rules of
  *   kmq_pack).  Codebook rows must be non-decreasing (otherwise the indices are
