@@ -11,11 +11,11 @@
 // memory, which adds them, applies the b = 1 codebook and stores bf16.
 //
 // The weights are rebuilt in registers (Dec1, Dec2, Dec4).  At b = 4 that costs 2.6 integer instructions a weight, and up
-// to 16 batch rows the integer pipe bounded the kernel (72 % busy, the shared-memory port 28 %): there the upper 8 rows of
-// a tile come from tables of all 256 (centroid, centroid) pairs in shared memory, half an instruction and half a load a
-// weight, and the lower 8 from registers, so that both pipes carry a part (8192 x 28672, us per call before / after:
-// M = 4 57.3 / 47.1, M = 16 65.0 / 54.2; 4096 x 4096, M = 16: 8.0 / 7.1).  With more batch rows the port is taken by the
-// activations' fragments.
+// to 16 batch rows the integer pipe bounded the kernel: there the upper 8 rows of a tile come from tables of all 256
+// (centroid, centroid) pairs in shared memory, half an instruction and half a load a weight, and the lower 8 from
+// registers, so that both pipes carry a part (8192 x 28672, us per call before / after: M = 4 57.3 / 47.1, M = 16
+// 65.0 / 54.2; 4096 x 4096, M = 16: 8.0 / 7.1; at M = 16 the integer pipe is now 53 % busy and the shared-memory port 60 %).
+// With more batch rows the port is taken by the activations' fragments.
 #include <atomic>
 
 #include "kmq_common.cuh"

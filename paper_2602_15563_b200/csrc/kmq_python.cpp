@@ -8,7 +8,7 @@
 //
 // torch tensors go through torch's DLPack exchange table (a C function per tensor, and one for the current stream); what
 // it does not describe, or another tensor library's object, is asked for data_ptr() instead.  Built against a torch whose
-// headers do not have the table (it came with DLPack 1.3; 2.11 has it), everything is.
+// headers do not have the table (it came with DLPack 1.3; 2.11 has it), everything is: 7.5 instead of 3.1 us a call.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 

@@ -12,9 +12,10 @@
 // (b = 8: two single lookups).  In the block format the table is the same for all rows, and the four MMAs of a group
 // make the unscaled sum of a block, which is scaled once in fp32: an exact product of scale and centroid does not fit a
 // bf16 operand, so both scale orders of the interface are evaluated this way; they differ by fp32 rounding only.
-// What bounds it: the lookups and their addresses, 8 integer instructions and 4 shared loads per 256 weights, next to
-// NT MMAs; on short rows the latency of a few dependent loads.  4096 x 4096, block format, b = 4, M = 8: 30 us on the
-// FMA units (2 passes over the weights, 5 instructions per weight).
+// What bounds it: the load port (lookups, 4 per 256 weights, and operands of which a load brings 16 bytes a lane to 4
+// lanes a row: 77 % busy on 8192 x 8192, block format, b = 4, M = 8, the integer pipe 24 %) and the latency of the loads
+// that a batch of groups waits for; on short rows that latency alone.  4096 x 4096, block format, b = 4, M = 8: 7.0 us, 30
+// on the FMA units before (2 passes over the weights, 5 instructions per weight).
 #include "kmq_rows.cuh"
 
 #include "kmq_mma_common.cuh"

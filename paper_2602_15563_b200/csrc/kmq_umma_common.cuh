@@ -1,4 +1,4 @@
-// Pieces shared by the tcgen05 kernels of kmq_linear (kmq_linear_umma.cu, kmq_linear_umma_pair.cu): mbarriers with
+// Pieces shared by the tcgen05 kernels of kmq_linear (kmq_linear_umma.cu, kmq_linear_umma_pair.cuh): mbarriers with
 // bounded waits, TMA tile loads of the activations, the tcgen05 instructions, the decode of packed words into tensor
 // memory.
 #pragma once
