@@ -15,7 +15,7 @@ namespace {
 
 // The scratch itself: part of the library's device image, present on every GPU that loads the library until the
 // process exits.  On GPUs with up to 160 SMs 640 KiB cover the balanced pair of one or two batch rows (3 * 1088 bytes per
-// SM) and the balanced form of the multi-tile kernel with 8 tiles per SM and up to 8 rows (4096 bytes per SM).
+// SM) and the balanced form of the multi-tile kernel with 4 tiles per SM and up to 8 rows (4096 bytes per SM).
 constexpr size_t kStaticScratchBytes = 640u * 1024u;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
