@@ -13,9 +13,17 @@
 //   * the producer thread copies the activations under a stage (NB batch rows x 128, zero-filled past M and past K)
 //     with two TMA tile loads (cp.async.bulk.tensor, 64 columns = 128 bytes wide, 128-byte swizzle) into a ring of B
 //     buffers with barriers of its own;
-//   * the MMA thread waits for both, issues 8 tcgen05.mma (128 x NB x 16 each) that add into the accumulator
+//   * the MMA thread waits for both, issues 8 tcgen05.mma (128 x NB x 16 each) that add into the accumulators
 //     D[128 output rows][NB batch rows], and commits them to the slots' `empty` barriers, which the decoders and the
 //     producer wait for before they overwrite the A operand and the B buffer.
+// A tcgen05.mma cuts its sum off instead of rounding it, so the error of a result grows with the number of MMAs that add into
+// one accumulator.  The slices of K therefore take turns on 2 to 8 accumulators (kAccs), which the epilogue adds: what fits
+// tensor memory beside enough A operands.  Share of results that are not the rounded exact ones, one accumulator / now
+// (mma.sync with its four or more chains, for comparison): 8192 x 28672, b = 4, M = 16 0.0080 / 0.0012 (0.0031); 12288 x 8192,
+// b = 4, M = 24 0.0042 / 0.0011 (0.0014); 4096 x 4096, b = 2, M = 40 0.00056 / 0.00030 (0.00037); 4096 x 2048, b = 2,
+// M = 128 0.00065 / 0.00032 (0.00039).  It costs up to 2 % up to 64 batch rows (8192 x 28672, b = 1, M = 16 28.15 -> 28.28 us),
+// 4 % up to 96 and up to 6 % with 128 (8192 x 28672, b = 1, M = 128 44.5 -> 46.1, 4096 x 1024, b = 4 6.5 -> 6.9), where it
+// leaves 4 stages in flight instead of 5.
 // b = 4, up to 64 batch rows: a row's 256 (centroid, centroid) pairs sit in shared memory, one bank per row, so that two
 // weights cost one PRMT and one conflict-free load (in registers: 5 integer instructions).  A tcgen05.mma of up to 64
 // batch rows takes 45 clocks, its 2048 weights 32 clocks of the load port, 16 of the integer pipe.
@@ -54,10 +62,14 @@ constexpr int exchange_columns(int nb) {
 template <int BITS, int NB>
 struct USmem {
   static constexpr bool kTab = BITS == 4 && NB <= 64;               // pair tables in shared memory
-  // stages in flight: A operands in tensor memory beside the accumulator, B buffers in shared memory beside the tables
-  static constexpr int kRing = NB <= 64 ? 7 - (kTab && NB > 32) : NB <= 96 ? 6 : 5;
+  static constexpr int kAccs = NB <= 16 ? 8 : NB <= 32 ? 4 : 2;     // accumulators of NB columns ...
+  static constexpr int kAccStride = NB == 48 ? 64 : NB;             // ... that many columns apart
+  // stages in flight: A operands in tensor memory beside the accumulators (and so B buffers in shared memory)
+  static constexpr int kRing = NB <= 64 ? 6 : NB <= 96 ? 5 : 4;
   static constexpr int kTmemCols = 512;
-  static_assert(kRing * 64 + NB <= 512, "tensor memory has 512 columns");
+  static_assert(kRing * 64 + kAccs * kAccStride <= 512, "tensor memory has 512 columns");
+  static_assert(UGeo<BITS>::kKSlices % kAccs == 0, "every stage adds to all accumulators");
+  static_assert(kRing >= kGroups, "a slot belongs to one group at a time");
   static constexpr int kBHalfBytes = NB * 128;                      // NB rows x 64 activations (one TMA box)
   static constexpr int kBStageBytes = 2 * kBHalfBytes;
   static constexpr int kB = 0;
@@ -65,9 +77,9 @@ struct USmem {
   static constexpr int kBars = kTables + (kTab ? 2 * 65536 : 0);    // full[kRing], empty[kRing], done
   static constexpr int kTmemSlot = kBars + (2 * kRing + 2) * 8;
   // Sums that the CTAs of a cluster hand over, columns of 128 floats.  Where they do not fit beside the rest they lie over
-  // the B buffers.
+  // the B buffers; with 128 batch rows too, where that is faster (1024 x 3072, b = 1, M = 128 8.1 us, beside the rest 8.6).
   static constexpr int kExchangeBytes = exchange_columns(NB) * kBM * 4;
-  static constexpr bool kOwnExchange = kTmemSlot + 16 + kExchangeBytes + 1024 <= 227 * 1024;
+  static constexpr bool kOwnExchange = NB <= 96 && kTmemSlot + 16 + kExchangeBytes + 1024 <= 227 * 1024;
   static constexpr int kExchange = kOwnExchange ? kTmemSlot + 16 : kB;
   static_assert(kOwnExchange || kExchangeBytes <= kBars, "the exchange lies over buffers that are free by then");
   static constexpr int kTotal = kTmemSlot + 16 + (kOwnExchange ? kExchangeBytes : 0) + 1024;   // + room to align the base
@@ -233,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  const uint32_t tmem_d = tmem_base + kRing * G::kCols;   // the accumulator follows the A operands
+  const uint32_t tmem_d = tmem_base + kRing * G::kCols;   // the accumulators follow the A operands
   asm volatile("griddepcontrol.launch_dependents;");
   if (SM::kOwnExchange && ksplit > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
@@ -247,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
         if (i >= total) break;
         if (round > 0) {
           // The MMAs of stage i - kRing are done: the slot may be overwritten.  (A wait by parity needs the phase before
-          // to be complete: that of stage i - 2 kRing, and this group has waited for stage i - 4 - kRing, a later one.)
+          // to be complete: that of stage i - 2 kRing, and this group has waited for stage i - 4 - kRing, no earlier one.)
           asm volatile("griddepcontrol.wait;" ::: "memory");
           ok = mbar_wait(empty_bar + 8 * slot, (round - 1) & 1);
           ok = __all_sync(0xFFFFFFFFu, ok);
@@ -298,7 +310,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
 #pragma unroll
       for (int ks = 0; ks < G::kKSlices; ++ks) {   // 16 activations = 32 bytes further inside a 128-byte row
         const uint32_t lo = desc_lo + (ks >> 2) * (SM::kBHalfBytes >> 4) + (ks & 3) * 2;
-        umma_bf16_elect(tmem_d, a_tmem + ks * 8, ((uint64_t)desc_hi << 32) | lo, idesc, ks > 0 || i > 0);
+        umma_bf16_elect(tmem_d + ks % SM::kAccs * SM::kAccStride, a_tmem + ks * 8, ((uint64_t)desc_hi << 32) | lo, idesc,
+                        ks >= SM::kAccs || i > 0);
       }
       umma_commit_elect(empty_bar + 8 * slot);
       if (++slot == kRing) {
@@ -344,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
 #pragma unroll 1
     for (int c = 8 * group; c < NB; c += 8 * kGroups) {
       uint32_t w[8];
-      load_acc<8>(w, tmem_d + ((uint32_t)(q * 32) << 16) + c, total > 0);
+      load_acc<SM::kAccs>(w, tmem_d + ((uint32_t)(q * 32) << 16) + c, SM::kAccStride, total > 0);
       if (ksplit > 1) {
         int owner = c / share, mine = c % share;
         const uint32_t here = smem_base + SM::kExchange + (rank * share * kBM + rho) * 4;

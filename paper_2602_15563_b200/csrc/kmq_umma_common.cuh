@@ -105,22 +105,35 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
-// This thread's lane of the accumulator, columns [col0, col0 + NC): all loads are issued before the one wait
-// (zeros when nothing was accumulated).
-template <int NC>
-__device__ __forceinline__ void load_acc(uint32_t (&w)[NC], uint32_t taddr, bool valid) {
-  static_assert(NC % 8 == 0, "whole groups of 8 columns");
+// This thread's lane of 8 columns from `taddr` on, added up over ACCS accumulators that lie `stride` columns apart (zeros when
+// nothing was accumulated).  All loads are issued before the one wait; their registers pass through an empty statement behind
+// it, so that no use of them is moved ahead of it.
+template <int ACCS>
+__device__ __forceinline__ void load_acc(uint32_t (&w)[8], uint32_t taddr, int stride, bool valid) {
   if (valid) {
+    uint32_t r[ACCS][8];
 #pragma unroll
-    for (int c = 0; c < NC; c += 8)
+    for (int a = 0; a < ACCS; ++a)
       asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(w[c + 0]), "=r"(w[c + 1]), "=r"(w[c + 2]), "=r"(w[c + 3]), "=r"(w[c + 4]), "=r"(w[c + 5]),
-                     "=r"(w[c + 6]), "=r"(w[c + 7])
-                   : "r"(taddr + c));
+                   : "=r"(r[a][0]), "=r"(r[a][1]), "=r"(r[a][2]), "=r"(r[a][3]), "=r"(r[a][4]), "=r"(r[a][5]), "=r"(r[a][6]),
+                     "=r"(r[a][7])
+                   : "r"(taddr + a * stride));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int a = 0; a < ACCS; ++a)
+      asm volatile("" : "+r"(r[a][0]), "+r"(r[a][1]), "+r"(r[a][2]), "+r"(r[a][3]), "+r"(r[a][4]), "+r"(r[a][5]),
+                        "+r"(r[a][6]), "+r"(r[a][7])::"memory");
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+#pragma unroll
+      for (int n = ACCS; n > 1; n /= 2)
+#pragma unroll
+        for (int a = 0; a < n / 2; ++a) r[a][j] = __float_as_uint(__uint_as_float(r[a][j]) + __uint_as_float(r[a + n / 2][j]));
+      w[j] = r[0][j];
+    }
   } else {
 #pragma unroll
-    for (int j = 0; j < NC; ++j) w[j] = 0;
+    for (int j = 0; j < 8; ++j) w[j] = 0;
   }
 }
 
