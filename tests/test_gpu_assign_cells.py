@@ -81,3 +81,14 @@ def test_weights_aligned_to_16_bytes_only(bits):
         kmq.kmq_block_quantize(W, N, K, bits, kmq.KMQ_LAMBDA_ABSMAX, 20, 4096, scales, shared, wq, sample)
         results.append([t.clone() for t in (cb, packed, scales, shared, wq)])
     assert all(torch.equal(a, b) for a, b in zip(*results))
+
+
+@pytest.mark.parametrize("K", (248, 256, 264))
+@pytest.mark.parametrize("layout", (kmq.KMQ_LAYOUT_CANONICAL, kmq.KMQ_LAYOUT_TUNED))
+def test_rows_at_the_length_from_which_cells_are_used(K, layout):
+    W = (np.random.default_rng(K).standard_normal((37, K)) * 0.02).astype(np.float32)
+    cb = torch.empty((37, 16), dtype=torch.bfloat16, device="cuda")
+    packed = torch.empty(kmq.kmq_packed_bytes(37, K, 4, layout) // 4, dtype=torch.int32, device="cuda")
+    kmq.kmq_quantize_rows(torch.from_numpy(W).cuda(), 37, K, 4, 20, layout, cb, packed)
+    got = gu.gpu_unpack(packed, 37, K, 4, layout)
+    assert np.array_equal(got, qorc.nearest_centroid(W, cb.view(torch.int16).cpu().numpy().view(np.uint16)))
