@@ -230,6 +230,9 @@ size_t kmq_static_scratch_capacity(void);
  * and from M = 9 on unless rows are short and few
  * (kmq_linear_variant() then starts with "tcgen05"); this entry point forces
  * it for any shape.
+ * packed and codebooks may be read before earlier work on `stream` has
+ * finished, as by kmq_linear, with the same condition on the kernel that
+ * writes them.
  * It needs no workspace.  Its waits on hardware barriers are bounded, see
  * kmq_device_error_flags.
  * Errors: KMQ_ERR_NULL, KMQ_ERR_BITS, KMQ_ERR_SHAPE, KMQ_ERR_ALIGN,

@@ -26,10 +26,10 @@ def in_turn(step, sync):
     return outs
 
 
-def weights(seed):
+def weights(seed, M=2):
     g = torch.Generator(device="cuda").manual_seed(seed)
     W = [torch.randn(N, K, device="cuda", generator=g) * (0.02 * (i + 1)) for i in range(ROUNDS)]
-    return W, torch.randn(2, K, device="cuda", generator=g).to(torch.bfloat16)
+    return W, torch.randn(M, K, device="cuda", generator=g).to(torch.bfloat16)
 
 
 def check(step):
@@ -54,6 +54,29 @@ def test_quantize_rows_then_linear(bits, layout):
     def step(i):
         kmq.kmq_quantize_rows(W[i], N, K, bits, 5, layout, cb, packed)
         kmq.kmq_linear(packed, cb, x, y[i], N, K, bits, M, ws, nbytes, layout=layout)
+        return y[i].clone()
+
+    check(step)
+
+
+@pytest.mark.parametrize("bits", (1, 2, 4))
+@pytest.mark.parametrize("M", (12, 40, 100, 200))
+@pytest.mark.parametrize("forced", (False, True))
+def test_quantize_rows_then_tcgen05(bits, M, forced):
+    """The kernel that reads packed words and codebooks of 128 rows ahead of its wait, by kmq_linear's choice and by its own
+    entry point."""
+    W, x = weights(20 + bits, M)
+    assert kmq.kmq_linear_variant(N, K, bits, M, T).startswith("tcgen05") and kmq.kmq_workspace_bytes(N, K, bits, M, T) == 0
+    packed = torch.zeros(kmq.kmq_packed_bytes(N, K, bits, T) // 4, dtype=torch.int32, device="cuda")
+    cb = torch.zeros(N, 1 << bits, dtype=torch.bfloat16, device="cuda")
+    y = torch.zeros(ROUNDS, M, N, dtype=torch.bfloat16, device="cuda")
+
+    def step(i):
+        kmq.kmq_quantize_rows(W[i], N, K, bits, 5, T, cb, packed)
+        if forced:
+            kmq.kmq_linear_tcgen05(packed, cb, x, y[i], N, K, bits, M)
+        else:
+            kmq.kmq_linear(packed, cb, x, y[i], N, K, bits, M, None, 0, layout=T)
         return y[i].clone()
 
     check(step)
