@@ -36,7 +36,17 @@ def test_kernel_on_either_side_of_a_line(bits, N, K, M, kernel):
     check(bits, N, K, M)
 
 
-# stages of 128 weights around the ring's 4 to 7 and the 4 groups of decoders; K that is no whole number of stages
+@pytest.mark.parametrize("bits,N,K,M", [(4, 10230, 8192, 16), (4, 8200, 28672, 9), (2, 10240, 8192, 32), (4, 2050, 28680, 12),
+                                        (2, 5130, 16400, 40), (2, 256, 512, 129), (2, 16, 64, 300), (2, 129, 640, 161),
+                                        (2, 1000, 1024, 520)])
+def test_shapes_that_had_another_kernel(bits, N, K, M):
+    """Once balanced shapes of the multi-tile kernel and shapes of the CTA pairs."""
+    (name, *_), = gu.linear_kernels(N, K, bits, M, TUNED)
+    assert template(name, "linear_umma_kernel")[0] == bits
+    check(bits, N, K, M)
+
+
+# stages of 128 weights around the rings of 4 to 6 and the 4 groups of decoders; K that is no whole number of stages
 @pytest.mark.parametrize("bits", (1, 2, 4))
 @pytest.mark.parametrize("K", (128, 384, 640, 768, 800, 896, 1024, 1152, 1312, 2016))
 @pytest.mark.parametrize("M", (40, 64, 90, 128))
