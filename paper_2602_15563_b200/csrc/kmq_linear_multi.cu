@@ -1,5 +1,5 @@
-// kmq_linear on the tuned (tile-major) layout for batches of up to 32 rows per launch (chosen from 2 to 9 rows
-// on, see linear_multi_min_rows, up to where linear_umma_selected takes over): the tiles of a CTA share the staged
+// kmq_linear on the tuned (tile-major) layout for batches of up to 32 rows (chosen from 2 to 9 rows on, see
+// linear_multi_min_rows, up to where linear_umma_selected takes over): the tiles of a CTA share the staged
 // activations, and the decode of a weight fragment is paid once and reused by up to 4 MMAs (one per group of 8 batch rows).
 //
 // One CTA owns TPC = 4 (or 2) tiles of 16 output rows.  Its 8 warps are 8 / TPC K-groups of TPC warps; warp
@@ -13,8 +13,7 @@
 // The weights are rebuilt in registers (Dec1, Dec2, Dec4).  At b = 4 that costs 2.6 integer instructions a weight, and up
 // to 16 batch rows the integer pipe bounded the kernel: there the upper 8 rows of a tile come from tables of all 256
 // (centroid, centroid) pairs in shared memory, half an instruction and half a load a weight, and the lower 8 from
-// registers, so that both pipes carry a part (8192 x 28672, us per call before / after: M = 4 57.3 / 47.1, M = 16
-// 65.0 / 54.2; 4096 x 4096, M = 16: 8.0 / 7.1; at M = 16 the integer pipe is now 53 % busy and the shared-memory port 60 %).
+// registers, so that both pipes carry a part (8192 x 28672, M = 4, us per call before / after: 57.3 / 47.1).
 // With more batch rows the port is taken by the activations' fragments.
 #include <atomic>
 
@@ -83,11 +82,11 @@ __device__ __forceinline__ void store_sums(const float (&v)[4], uint16_t* __rest
   }
 }
 
-// Resident CTAs per SM that the register budget is for (two of 8 warps fit up to 32 batch rows, but only the balanced form,
+// Resident CTAs per SM that the register budget is for (two of 8 warps fit up to 16 batch rows, but only the balanced form,
 // whose loop over the groups makes the compiler generous, needs to be told with 4 tiles).
 template <int NT, int TPC, int W, bool SPLIT>
 constexpr int multi_ctas_per_sm() {
-  return W == 8 && (SPLIT ? NT <= 4 : NT <= 2 && TPC == 2) ? 2 : 1;
+  return W == 8 && (SPLIT || (NT <= 2 && TPC == 2)) ? 2 : 1;
 }
 
 // SPLIT: the balanced form.  The (group of TPC tiles, step) units, group by group, are cut into gridDim.x equal ranges,
@@ -364,14 +363,18 @@ struct MultiCall {
   cudaStream_t s;
 };
 
-template <int BITS, int NT, int TPC, int W = 8>
+// BALANCED: this shape of CTA has a balanced form.
+template <int BITS, int NT, int TPC, int W = 8, bool BALANCED = true>
 cudaError_t launch_nt(const MultiCall& c) {
   constexpr int smem = MSmem<BITS, NT, TPC, W>::kTotal;
   const int64_t tiles = (c.N + kTileRows - 1) / kTileRows, groups = (tiles + TPC - 1) / TPC;
-  const DeviceInfo* di = device_info();
-  if (!di) return cudaErrorInvalidDevice;
-  const int slots = di->sm_count * resident_ctas<BITS, NT, TPC, W>();
-  if (slots <= 0) return cudaErrorInvalidConfiguration;
+  int slots = 0;
+  if constexpr (BALANCED) {
+    const DeviceInfo* di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    slots = di->sm_count * resident_ctas<BITS, NT, TPC, W>();
+    if (slots <= 0) return cudaErrorInvalidConfiguration;
+  }
   if (c.plan) {
     c.plan->ctas = slots;
     c.plan->tiles = TPC;
@@ -388,9 +391,8 @@ cudaError_t launch_nt(const MultiCall& c) {
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  const unsigned grid = c.scratch ? (unsigned)slots : (unsigned)groups;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3((unsigned)groups);
   cfg.blockDim = dim3(W * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c.s;
@@ -399,16 +401,21 @@ cudaError_t launch_nt(const MultiCall& c) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (!c.scratch)
-    return cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, false>, c.packed, c.cb, c.x, c.y, c.N, c.K, c.M,
-                              c.scratch);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, true>, c.packed, c.cb, c.x, c.y, c.N, c.K,
-                                     c.M, c.scratch);
-  if (e != cudaSuccess) return e;
-  cfg.gridDim = dim3((unsigned)groups, TPC);
-  cfg.blockDim = dim3(32 * NT);
-  cfg.dynamicSmemBytes = 0;
-  return cudaLaunchKernelEx(&cfg, linear_multi_sum_kernel<BITS, NT, TPC>, (const float*)c.scratch, c.y, c.N, c.K, c.M, slots);
+  if constexpr (BALANCED) {
+    if (c.scratch) {
+      cfg.gridDim = dim3((unsigned)slots);
+      cudaError_t e = cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, true>, c.packed, c.cb, c.x, c.y, c.N, c.K,
+                                         c.M, c.scratch);
+      if (e != cudaSuccess) return e;
+      cfg.gridDim = dim3((unsigned)groups, TPC);
+      cfg.blockDim = dim3(32 * NT);
+      cfg.dynamicSmemBytes = 0;
+      return cudaLaunchKernelEx(&cfg, linear_multi_sum_kernel<BITS, NT, TPC>, (const float*)c.scratch, c.y, c.N, c.K, c.M,
+                                slots);
+    }
+  }
+  return cudaLaunchKernelEx(&cfg, linear_multi_kernel<BITS, NT, TPC, W, false>, c.packed, c.cb, c.x, c.y, c.N, c.K, c.M,
+                            (float*)nullptr);
 }
 
 template <int BITS>
@@ -416,13 +423,13 @@ cudaError_t launch_bits(const MultiCall& c) {
   const int64_t N = c.N, K = c.K;
   const int M = c.M;
   // Tiles per CTA: 4 share the staged activations among more warps, 2 give twice as many CTAs.  Measured: 2 wins
-  // when 4 would leave more than half of the SMs without a CTA, and for b = 2, 4 at up to 16 rows (two CTAs then fit an SM).
+  // when 4 would leave more than half of the SMs without a CTA, and for b = 2, 4 (two CTAs then fit an SM).
   const DeviceInfo* di = device_info();
   const int64_t tiles = (N + kTileRows - 1) / kTileRows;
   const bool few = (tiles + 3) / 4 <= (di ? di->sm_count : 148) / 2;
   const bool fits_one_wave = (tiles + 3) / 4 <= (di ? di->sm_count : 148);   // CTAs of 4 tiles <= SMs
   // few tiles and a long K: 2 tiles x 8 K-groups (16 warps) while each K-group still gets 4 steps or more
-  // (4096 x 11008, b = 2, M = 16: 13.4 -> 12.3 us; 4096 x 4096: b = 4 11.5 -> 9.8 us, b = 2 (16 steps) 6.4 -> 6.9 us)
+  // (4096 x 11008, b = 2, M = 6: 13.4 -> 9.0 us; 4160 x 4096, b = 4, M = 7 7.8 -> 5.9; 4096 x 11008, b = 1, M = 8 12.1, 12.2)
   const bool few16 = few && (tiles + 1) / 2 <= (di ? di->sm_count : 148) && tuned_row_steps(K, BITS) >= 32;
   if (M <= 8) {
     // same shape of CTA for up to 8 batch rows (8192 x 28672, b = 1, M = 4: 35.0 -> 23.5 us; 8192 x 8192, b = 2,
@@ -434,34 +441,27 @@ cudaError_t launch_bits(const MultiCall& c) {
     if (few || BITS != 1) return launch_nt<BITS, 1, 2>(c);
     return launch_nt<BITS, 1, 4>(c);
   }
+  // More rows: what linear_umma_selected leaves.  Where a driver has no tensor-map encoder, all calls of more rows are made with
+  // these forms, which serve any shape.
   if (M <= 16) {
-    // 4 tiles x 4 K-groups (16 warps) when that grid gives every SM at most one CTA: 8192 x 8192, b = 2, M = 16:
-    // 16.1 -> 14.4 us; 8192 x 28672, M = 16: b = 1 47.9 -> 40.1 us, b = 4 85.2 -> 76.6 us
-    if (!few && fits_one_wave) return launch_nt<BITS, 2, 4, 16>(c);
-    if constexpr (MSmem<BITS, 2, 2, 16>::kTotal <= kMaxSmem) {
-      if (few16) return launch_nt<BITS, 2, 2, 16>(c);
+    if constexpr (BITS == 1) {
+      if (!few) return launch_nt<BITS, 2, 4>(c);
+    } else if constexpr (BITS == 4) {   // 6000 x 768, M = 12 4.0 -> 3.2 us, 9000 x 896, M = 16 5.1 -> 3.9
+      if (!few && fits_one_wave) return launch_nt<BITS, 2, 4, 16, false>(c);
     }
-    if (few || BITS != 1) return launch_nt<BITS, 2, 2>(c);
-    return launch_nt<BITS, 2, 4>(c);
+    return launch_nt<BITS, 2, 2, 8, false>(c);
   }
-  if (M <= 32) {
-    if constexpr (MSmem<BITS, 4, 2>::kTotal <= kMaxSmem) {
-      if (few) return launch_nt<BITS, 4, 2>(c);
-    }
-    // when every SM gets at most one CTA anyway: 4 K-groups, i.e. 16 warps per CTA instead of 8 (8192 x 8192,
-    // b = 2, M = 32: 22.6 -> 20.3 us; with more CTAs than SMs two 8-warp CTAs share an SM and that is faster)
-    if constexpr (MSmem<BITS, 4, 4, 16>::kTotal <= kMaxSmem) {
-      if (fits_one_wave) return launch_nt<BITS, 4, 4, 16>(c);
-    }
-    return launch_nt<BITS, 4, 4>(c);
+  if constexpr (BITS != 1) {
+    if (M <= 32) return launch_nt<BITS, 4, 2, 8, false>(c);
   }
-  return cudaErrorInvalidValue;   // unreachable: launched in passes of at most 32 rows
+  return cudaErrorInvalidValue;   // unreachable: launched in passes of linear_multi_rows_per_launch() rows
 }
 
 }  // namespace
 
-// Batch rows per launch of the multi-tile kernel (more than that come here only where the tcgen05 kernel can not run).
-int linear_multi_rows_per_launch() { return 32; }
+// Batch rows per launch of the multi-tile kernel: what its forms take (at b = 1 the activations under a step of 32 rows do not
+// fit shared memory).  More than that come here only where the tcgen05 kernel can not run.
+int linear_multi_rows_per_launch(int bits) { return bits == 1 ? 16 : 32; }
 
 // Smallest batch that goes to the multi-tile kernel.  The GEMV kernel stages the activations once per tile, here the tiles
 // of a CTA share them; but its grid is finer, and it shares K among a cluster.  The lines below are from a sweep of 20 to
@@ -521,22 +521,21 @@ static cudaError_t launch_multi(int bits, const MultiCall& c) {
 //          M = 8 12.0 / 12.2; 6400 x 8192, 170, 15.5 / 15.3), 140 where the groups nearly fill the SMs, so that few are
 //          shared by more than two CTAs (8192 x 16384, 142, M = 3 28.4 / 28.6, M = 8 29.5 / 29.4; 8192 x 20480, 177,
 //          M = 8 36.0 / 35.0).
-//   more   some 9000 clocks, of which an SM does 20 weights each (24 at b = 2), 12 with more than 16 rows.  8192 x 28672,
-//          M = 16 (128 groups on 148 slots): b = 4 53.9 / 51.2, b = 2 42.6 / 39.1; 10240 x 8192 (320 on 296): b = 4,
-//          M = 16 32.5 / 25.6, b = 2, M = 32 43.4 / 28.3; but 8192 x 8192, b = 4, M = 16 17.6 / 20.2, 12288 x 4096, b = 2,
-//          M = 12 12.9 / 13.5.
+//   more   at b = 1, 4 tiles a CTA, the only calls of more rows here that leave slots empty on long rows: 180 (14080 x 8192,
+//          M = 16 23.4 / 21.2; 9600 x 16384 42.6 / 26.9).
 MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
   MultiSplit sp = {};
   const DeviceInfo* di = device_info();
-  if (!di || M > linear_multi_rows_per_launch()) return sp;
-  if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess) return {};
+  if (!di || M > linear_multi_rows_per_launch(bits)) return sp;
+  if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess || sp.ctas == 0)
+    return {};
   const int64_t steps = tuned_row_steps(K, bits), sms = di->sm_count;
   // CTAs that have an SM to themselves run as fast as the SM lets them: then it is the SMs that are empty, not the slots
   const int64_t slots = sp.groups <= sms ? sms : sp.ctas, waves = (sp.groups + slots - 1) / slots;
   const double saved = (double)(waves * slots - sp.groups) / slots * (double)steps;
   const double weights = saved * (double)(slots / sms) * sp.tiles * (kTileRows * 512 / bits);   // of one SM
   double cost;
-  if (M > 8) cost = 9000.0 * (M > 16 ? 12.0 : bits == 2 ? 24.0 : 20.0);
+  if (M > 8) cost = 180e3;
   else if (bits == 4) cost = sp.groups <= sms && 6 * sp.groups >= 5 * sms ? 140e3 : 165e3;
   else cost = bits == 1 ? 190e3 : waves > 1 ? 340e3 : 172e3;
   return weights > cost && sp.groups * steps >= sp.ctas ? sp : MultiSplit{};
@@ -544,7 +543,7 @@ MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
 
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s) {
-  const int64_t per = linear_multi_rows_per_launch();
+  const int64_t per = linear_multi_rows_per_launch(bits);
   for (int64_t m0 = 0; m0 < M; m0 += per) {
     const int mc = (int)(M - m0 < per ? M - m0 : per);
     const uint16_t* xp = x + m0 * K;
