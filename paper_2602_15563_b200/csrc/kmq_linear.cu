@@ -39,7 +39,7 @@ LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout, si
     return p;
   }
   if (M >= linear_multi_min_rows(bits, N, K)) {
-    const int64_t per = linear_multi_rows_per_launch(bits);
+    const int64_t per = linear_multi_rows_per_launch();
     p.variant = kVariantMulti;
     p.launches = (int)((M + per - 1) / per);
     p.name = bits == 4 ? "multi_prmt_b4" : bits == 2 ? "multi_prmt_b2" : "multi_select_b1";

@@ -451,17 +451,15 @@ cudaError_t launch_bits(const MultiCall& c) {
     }
     return launch_nt<BITS, 2, 2, 8, false>(c);
   }
-  if constexpr (BITS != 1) {
-    if (M <= 32) return launch_nt<BITS, 4, 2, 8, false>(c);
-  }
+  // b = 1 (only without the encoder): 4 K-groups of 2 tiles would need 278 KB for their activations
+  if (M <= 32) return launch_nt<BITS, 4, BITS == 1 ? 4 : 2, 8, false>(c);
   return cudaErrorInvalidValue;   // unreachable: launched in passes of linear_multi_rows_per_launch() rows
 }
 
 }  // namespace
 
-// Batch rows per launch of the multi-tile kernel: what its forms take (at b = 1 the activations under a step of 32 rows do not
-// fit shared memory).  More than that come here only where the tcgen05 kernel can not run.
-int linear_multi_rows_per_launch(int bits) { return bits == 1 ? 16 : 32; }
+// Batch rows per launch of the multi-tile kernel (more than that come here only where the tcgen05 kernel can not run).
+int linear_multi_rows_per_launch() { return 32; }
 
 // Smallest batch that goes to the multi-tile kernel.  The GEMV kernel stages the activations once per tile, here the tiles
 // of a CTA share them; but its grid is finer, and it shares K among a cluster.  The lines below are from a sweep of 20 to
@@ -526,7 +524,7 @@ static cudaError_t launch_multi(int bits, const MultiCall& c) {
 MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
   MultiSplit sp = {};
   const DeviceInfo* di = device_info();
-  if (!di || M > linear_multi_rows_per_launch(bits)) return sp;
+  if (!di || M > linear_multi_rows_per_launch()) return sp;
   if (launch_multi(bits, {nullptr, nullptr, nullptr, nullptr, N, K, (int)M, nullptr, &sp, nullptr}) != cudaSuccess || sp.ctas == 0)
     return {};
   const int64_t steps = tuned_row_steps(K, bits), sms = di->sm_count;
@@ -543,7 +541,7 @@ MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M) {
 
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s) {
-  const int64_t per = linear_multi_rows_per_launch(bits);
+  const int64_t per = linear_multi_rows_per_launch();
   for (int64_t m0 = 0; m0 < M; m0 += per) {
     const int mc = (int)(M - m0 < per ? M - m0 : per);
     const uint16_t* xp = x + m0 * K;

@@ -33,7 +33,7 @@ struct MultiSplit {     // the balanced form of the multi-tile kernel
   size_t scratch;
 };
 MultiSplit linear_multi_split(int64_t N, int64_t K, int bits, int64_t M);
-int linear_multi_rows_per_launch(int bits);
+int linear_multi_rows_per_launch();
 int linear_multi_min_rows(int bits, int64_t N, int64_t K);   // smallest batch routed to the multi-tile kernel
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s);   // scratch: balanced form
