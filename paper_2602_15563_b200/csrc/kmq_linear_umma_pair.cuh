@@ -1,6 +1,7 @@
 // kmq_linear on the tuned layout for prefill batches (M > 128): tcgen05.mma over a pair of CTAs.  Included by
-// kmq_linear_umma.cu, whose single-CTA kernel does the same for up to 128 batch rows; the roles of the warps, the ring of
-// packed words and the decode into tensor memory are that kernel's.
+// kmq_linear_umma.cu, whose single-CTA kernel does the same for up to 128 batch rows; the roles of the warps are that kernel's.
+// Here all 16 decoder warps rebuild every stage together, from packed words that a ring of cp.async copies brings to shared
+// memory, with a barrier of theirs per step (up to 256 batch rows per decode: the tensor core is what the others wait for).
 //
 // What bounds it: one SM multiplies 128 x 256 x 16 in 128 clocks, and the 256 activations rows of that step are 8 KB, so
 // a CTA on its own would draw 64 bytes per clock from L2, more than L2 gives 148 SMs at once; with 128 batch rows per
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) linear_umma_pair_kernel(const
   bool ok = true;
 
   if (warp < kDecodeWarps) {
-    // ================= decoder warps: as in linear_umma_kernel, on from tile to tile =================
+    // ================= decoder warps, on from tile to tile =================
     const int q = warp & 3, kh = warp >> 2;
     const int rho = 32 * q + lane;
     const int64_t row_tiles = (N + kTileRows - 1) / kTileRows;

@@ -56,7 +56,8 @@ struct Dec2 {
     lo = prmt(c.x, c.y, 0x6420u);
     hi = prmt(c.x, c.y, 0x7531u);
   }
-  // phase q of a word: fields q, q+4, q+8, q+12 -> (W_q, W_q+4) and (W_q+8, W_q+12)
+  // The indices at bits 2 q + 8 c of a word, c = 0 .. 3, as two pairs of weights, c = 0, 1 and c = 2, 3.  In the tuned layout
+  // they are the consecutive weights 4 q + c; in the canonical one the weights q + 4 c.
   __device__ __forceinline__ void pair(uint32_t w, int q, uint32_t& a_first, uint32_t& a_second) const {
     const uint32_t f = (w >> (2 * q)) & 0x03030303u;
     const uint32_t sel = f * 0x11u + 0x40404040u;   // per byte: nibbles (i, 4 + i) select (lo_i, hi_i)
