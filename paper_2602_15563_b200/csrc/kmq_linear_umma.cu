@@ -22,8 +22,8 @@
 // (mma.sync with its four or more chains, for comparison): 8192 x 28672, b = 4, M = 16 0.0080 / 0.0012 (0.0031); 12288 x 8192,
 // b = 4, M = 24 0.0042 / 0.0011 (0.0014); 4096 x 4096, b = 2, M = 40 0.00056 / 0.00030 (0.00037); 4096 x 2048, b = 2,
 // M = 128 0.00065 / 0.00032 (0.00039).  It costs up to 3 % up to 64 batch rows (8192 x 28672, b = 1, M = 16 28.15 -> 28.28 us;
-// 14000 x 1024, b = 4, M = 16 4.63 -> 4.78), 4 % up to 96 and up to 6 % with 128 (8192 x 28672, b = 1, M = 128 44.5 -> 46.1, 4096 x 1024, b = 4 6.5 -> 6.9), where it
-// leaves 4 stages in flight instead of 5.
+// 14000 x 1024, b = 4, M = 16 4.63 -> 4.78), 4 % up to 96 and up to 6 % with 128 (8192 x 28672, b = 1, M = 128 44.5 -> 46.1,
+// 4096 x 1024, b = 4 6.5 -> 6.9), where it leaves 4 stages in flight instead of 5.
 // b = 4, up to 64 batch rows: a row's 256 (centroid, centroid) pairs sit in shared memory, one bank per row, so that two
 // weights cost one PRMT and one conflict-free load (in registers: 5 integer instructions).  A tcgen05.mma of up to 64
 // batch rows takes 45 clocks, its 2048 weights 32 clocks of the load port, 16 of the integer pipe.
