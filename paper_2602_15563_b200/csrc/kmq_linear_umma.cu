@@ -123,6 +123,12 @@ __device__ __forceinline__ void tmem_store16(uint32_t taddr, const uint32_t (&v)
       "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
       : "memory");
 }
+// The loads of w are waited for here.
+template <int NW>
+__device__ __forceinline__ void arrived(uint32_t (&w)[NW]) {
+#pragma unroll
+  for (int i = 0; i < NW; i += 4) asm volatile("" : "+r"(w[i]), "+r"(w[i + 1]), "+r"(w[i + 2]), "+r"(w[i + 3]));
+}
 // Word(s) number `c` of a stage -> 32 weights as bf16 pairs in the order of k.  `bank`: this lane's place in the pair
 // tables, byte 1 open for an index byte.
 template <int BITS, int NW, bool TAB>
@@ -266,6 +272,15 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
           if (!ok) break;
           tc_fence_after_sync();
         }
+        // The words of the stage before are loaded anew only now that this stage's have arrived: a wait for registers of a load
+        // is a wait for later loads too, where they share one of a warp's few counters, and behind the stage's decode each
+        // round ended with the latency of the load just issued.  us, before / now: 8192 x 28672, M = 16, b = 4 29.4 / 28.1,
+        // b = 2 31.9 / 30.2; at b = 1, with eight loads of one word each in flight, 28.1 / 28.4.
+        if constexpr (BITS >= 2) {
+          arrived<NW>(words[p]);
+          if (i != group && i + (kAhead - 1) * kGroups < total)
+            load_stage(words[(p + kAhead - 1) % kAhead], i + (kAhead - 1) * kGroups);
+        }
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + slot * G::kCols;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -273,7 +288,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
           decode32<BITS, NW, SM::kTab>(a, words[p], c, st, tables, bank);
           tmem_store16(taddr + 16 * c, a);
         }
-        if (i + kAhead * kGroups < total) load_stage(words[p], i + kAhead * kGroups);
+        if constexpr (BITS == 1)
+          if (i + kAhead * kGroups < total) load_stage(words[p], i + kAhead * kGroups);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before_sync();
         __syncwarp();
