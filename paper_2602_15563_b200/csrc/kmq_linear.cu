@@ -31,7 +31,10 @@ LinearPlan plan_linear(int64_t N, int64_t K, int bits, int64_t M, int layout, si
     else p.name = bits == 4 ? "staged_pairtable_b4" : bits == 2 ? "staged_pairtable_b2" : "staged_pairtable_b1";
     return p;
   }
-  if (linear_umma_selected(N, K, bits, M)) {
+  // (the balanced pairs of kernels, whose callers bring scratch for them, keep their shapes)
+  const bool few = linear_umma_few_rows(N, K, bits, M) && !linear_split_ctas(N, K, bits, M) &&
+                   !(M >= linear_multi_min_rows(bits, N, K) && linear_multi_split(N, K, bits, M).ctas);
+  if (few || linear_umma_selected(N, K, bits, M)) {
     const int64_t per = linear_umma_rows_per_launch();
     p.variant = kVariantUmma;
     p.launches = (int)((M + per - 1) / per);

@@ -579,6 +579,35 @@ bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M) {
   return K >= 2048 || N >= 4096 || (bits == 1 && K <= 512);
 }
 
+// Which calls of up to 8 batch rows come here, of those that no balanced pair of kernels takes.  What decides is how the 128-row
+// blocks fill the machine and how the 16-row tiles do: the GEMV kernel at b = 4 has room for three tiles an SM (444, 7104 rows),
+// and is bound by its table port where this kernel decodes a quarter faster; rows must be long enough to pay for this kernel's
+// start.  Lines from a sweep of 16 x 13 shapes (256 to 16384 rows of 256 to 28672 weights) at 1, 2, 4 and 8 batch rows; us per
+// call, GEMV or multi-tile / this: b = 4, M = 1 8192 x 8192 15.2 / 11.9, 16384 x 8192 25.4 / 19.4, but 6144 x 6144 7.9 / 8.7 and
+// (blocks that fill 58 % of the machine and can not be split) 11008 x 4096 9.6 / 10.2; M = 8 14336 x 4096 17.9 / 11.3,
+// 3072 x 8192 8.9 / 7.2; b = 2, M = 8 16384 x 8192 23.4 / 19.3.
+// Between kernels of the other kind a call here costs some 2.4 us more (neither can set up beside the other): a decode step of
+// 3072 / 8192, b = 4, M = 1 took 345.7 us with its 16384 x 3072 layers here (11.7 / 9.4 by themselves) against 339.2.  Where the
+// gain is of that size a call stays where it was, hence the lines at 2^26 weights and at K = 2048 to 4096 (steps of 2048 / 5376,
+// b = 4, M = 4 233.7 us, with the 10752 x 2048 layers here 241.4; of 3072 / 8192, M = 4 260.7 / 227.4).
+bool linear_umma_few_rows(int64_t N, int64_t K, int bits, int64_t M) {
+  const DeviceInfo* di = device_info();
+  if (!di || M > 8 || !encode_tiled()) return false;
+  const int64_t sms = di->sm_count, blocks = (N + kBM - 1) / kBM, waves = (blocks + sms - 1) / sms;
+  if (blocks < 8) return false;                            // the GEMV kernel's clusters fill the machine with them
+  const int64_t filled = 100 * blocks / (waves * sms);     // % of the machine, one CTA a block
+  const bool half = 2 * blocks <= sms;                     // room for two CTAs a block
+  if (bits == 4 && M > 2) {
+    if (!half) return filled >= 64 ? K >= 2048 : filled >= 55 && K >= 4096;
+    if (blocks >= 53) return K >= (M <= 5 ? 6144 : 4096);
+    if (blocks >= 40) return K >= 3072;
+    return K >= (M <= 5 ? 8192 : 6144);
+  }
+  if (bits == 1 || N * K < (int64_t(1) << 26)) return false;
+  if (bits == 4) return !half ? filled >= 64 : blocks >= 56 || blocks <= 40;
+  return M >= 6 && filled >= 75;
+}
+
 // Whether more than 128 batch rows go to the CTA pairs (256 x 256 tiles, persistent).  Fitted as above, 5 % standard
 // deviation: us per call, pairs / batch tiles of 128 rows: 16384 x 3072, b = 2, M = 1024 95 / 164 (at the time the pairs
 // were written); 512 x 1280, b = 1, M = 256 15.3 / 7.2; 13184 x 6528, b = 4, M = 512 95.5 / 82.7.

@@ -10,7 +10,7 @@ enum LinearVariant : int {
   kVariantTiled = 2,     // tuned (tile-major) layout: tensor-core GEMV with coalesced 1 KB steps, small batches (M <= 8)
   kVariantMulti = 3,     // tuned layout, M >= linear_multi_min_rows(): 32 or 64 output rows per CTA share the staged
                          // activations, one decode feeds up to 4 MMAs
-  kVariantUmma = 5,      // tuned layout, M > 8 (linear_umma_selected()): tcgen05.mma, weights dequantised into tensor memory
+  kVariantUmma = 5,      // tuned layout (linear_umma_selected(), linear_umma_few_rows()): tcgen05.mma, weights dequantised into tensor memory
   kVariantSplit = 4,     // tuned layout, M <= 2, more tiles than resident CTAs: equal step ranges + fix-up (scratch)
   kVariantLut = 6,       // table layout, b = 1, 2: activation tables in shared memory, one lookup per 8 weights (scratch)
   kVariantUnsupported = 7,
@@ -38,6 +38,7 @@ int linear_multi_min_rows(int bits, int64_t N, int64_t K);   // smallest batch r
 cudaError_t launch_linear_multi(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
                                 int64_t K, int bits, int64_t M, void* scratch, cudaStream_t s);   // scratch: balanced form
 bool linear_umma_selected(int64_t N, int64_t K, int bits, int64_t M);   // kmq_linear's choice of the tcgen05 kernel
+bool linear_umma_few_rows(int64_t N, int64_t K, int bits, int64_t M);   // ... for up to 8 batch rows, where no balanced pair of kernels runs
 int64_t linear_umma_rows_per_launch();
 int linear_umma_ksplit(int64_t N, int64_t K, int bits, int64_t batch);   // CTAs (cluster size) per 128-row block
 cudaError_t launch_linear_umma(const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y, int64_t N,
