@@ -1,7 +1,9 @@
 // kmq_dequant_to_bf16: W^[n,k] = C_n[idx[n,k]] as a dense bf16 matrix.
-// The kernel is bound by the 2-byte-per-weight output stream, so every thread
-// produces exactly one 16-byte store (8 weights) from 8*BITS packed bits and
-// consecutive threads write consecutive 16-byte pieces.
+// The kernels are bound by the 2-byte-per-weight output stream.  A warp has a share of one row, up to kBatch x 32 chunks of
+// 8 weights: it loads the packed bits of all of them, then decodes and stores, 16 bytes a lane, consecutive lanes writing
+// consecutive pieces.  CTAs are short and many, dealt out by the hardware: SMs do not all reach memory equally fast, and a
+// grid that stays resident, with equal shares for all, ends with the slowest (470 MB of plain stores: 76.6 us from 1184 CTAs
+// in a loop, 64 to 68 us from 9472 and more).  8192 x 28672, b = 4 106.0 -> 92.4 us.
 #include "kmq_common.cuh"
 #include "kmq_table_layout.cuh"
 
@@ -53,113 +55,138 @@ __device__ __forceinline__ void load_codebook(const uint16_t* __restrict__ row_c
   if constexpr (BITS == 4) c0 = __ldg(row_cb + (threadIdx.x & 15));
 }
 
-// One CTA walks rows (grid-stride); inside a row every thread turns 8 weights into one 16-byte streaming store,
-// consecutive threads writing consecutive pieces.  In the tuned layout the row's words come in 64-byte runs, one
-// per 1 KB step of its tile, and the 8 fields of a chunk are cut out of the word after one shift.
+constexpr int kWarps = 8, kBatch = 4;
+
+// Shares of a row (in chunks of 8 weights) and the grid for N rows; CTAs beyond the largest grid are made up for by a loop.
+inline int row_shares(int64_t K) { return (int)((K / 8 + 32 * kBatch - 1) / (32 * kBatch)); }
+inline unsigned share_grid(int64_t N, int64_t K) {
+  const int64_t ctas = (N * row_shares(K) + kWarps - 1) / kWarps;
+  return (unsigned)(ctas < (int64_t(1) << 30) ? ctas : int64_t(1) << 30);
+}
+
+// f(row, first chunk) for every share of this warp.
+template <class F>
+__device__ __forceinline__ void for_each_share(int64_t N, int shares, F f) {
+  const int64_t all = N * shares;
+  for (int64_t t = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5); t < all; t += (int64_t)gridDim.x * kWarps) {
+    const int64_t n = all <= 0xFFFFFFFFll ? (int64_t)((uint32_t)t / (uint32_t)shares) : t / shares;
+    f(n, (int)(t - n * shares) * (32 * kBatch));
+  }
+}
+
+// In the tuned layout the row's words come in 64-byte runs, one per 1 KB step of its tile, and the 8 fields of a chunk are
+// cut out of the word after one shift.
 template <int BITS, bool TUNED>
-__global__ void __launch_bounds__(256) dequant_rows_kernel(const uint32_t* __restrict__ packed,
-                                                           const uint16_t* __restrict__ cb, uint16_t* __restrict__ W,
-                                                           int64_t N, int64_t K) {
+__global__ void __launch_bounds__(kWarps * 32) dequant_rows_kernel(const uint32_t* __restrict__ packed,
+                                                                   const uint16_t* __restrict__ cb,
+                                                                   uint16_t* __restrict__ W, int64_t N, int64_t K,
+                                                                   int shares) {
   constexpr int Q = 1 << BITS;
   constexpr int CPW = 4 / BITS;                  // 8-weight chunks per word
   const int cpr = (int)(K >> 3);                 // 8-weight chunks per row
   const int64_t wpr = K / (32 / BITS);           // words per row
   const int64_t steps = tuned_steps(wpr);
-  for (int64_t n = blockIdx.x; n < N; n += gridDim.x) {
+  for_each_share(N, shares, [&](int64_t n, int first) {
     const uint32_t* row_words =
         TUNED ? packed + ((n >> 4) * steps * kTileRows + (n & 15)) * 16 : packed + n * wpr;
     const uint16_t* row_cb = cb + n * Q;
     uint32_t c0, c1;
     load_codebook<BITS>(row_cb, c0, c1);
-    uint4* out = reinterpret_cast<uint4*>(W + n * K);
-    // b = 4 looks its centroids up by warp shuffles, so there whole warps stay in the loop (lanes past the end of
-    // the row decode a zero word and store nothing)
-    const int cend = BITS == 4 ? (cpr + 31) & ~31 : cpr;
-    for (int c = threadIdx.x; c < cend; c += 256) {
-      const bool live = BITS != 4 || c < cpr;
-      uint32_t v = 0;
-      if (!live) {
-      } else if constexpr (TUNED) {
-        const int j = c / CPW, q = c % CPW;
-        const uint32_t t = __ldg(row_words + (int64_t)(j >> 4) * 256 + (j & 15));
-        if constexpr (BITS == 4) {
-          v = t;
-        } else if constexpr (BITS == 2) {
-          // field 4p + c' at bits 2p + 8c'; chunk q holds p = 2q, 2q+1: shift them down to p = 0, 1
-          const uint32_t u = t >> (4 * q);
-          v = 0;
+    uint4* const out = reinterpret_cast<uint4*>(W + n * K);
+    const int c_lane = first + (threadIdx.x & 31);
+    uint32_t t[kBatch];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) v |= ((u >> field_pos<2>(i, true)) & 3u) << (2 * i);
-        } else {
-          // field 2c' at bit 15 - c', field 2c'+1 at bit 31 - c'; chunk q holds c' = 4q .. 4q+3
-          const uint32_t u = t << (4 * q);
-          v = 0;
+    for (int i = 0; i < kBatch; ++i) {
+      const int c = c_lane + 32 * i, j = c / CPW;
+      t[i] = 0;
+      if (c >= cpr) continue;
+      if constexpr (TUNED) t[i] = __ldg(row_words + (int64_t)(j >> 4) * 256 + (j & 15));
+      else if constexpr (BITS == 4) t[i] = __ldg(row_words + c);
+      else if constexpr (BITS == 2) t[i] = __ldg(reinterpret_cast<const uint16_t*>(row_words) + c);
+      else t[i] = __ldg(reinterpret_cast<const uint8_t*>(row_words) + c);
+    }
 #pragma unroll
-          for (int i = 0; i < 8; ++i) v |= ((u >> field_pos<1>(i, true)) & 1u) << i;
-        }
-      } else if constexpr (BITS == 4) {
-        v = __ldg(row_words + c);
-      } else if constexpr (BITS == 2) {
-        v = __ldg(reinterpret_cast<const uint16_t*>(row_words) + c);
-      } else {
-        v = __ldg(reinterpret_cast<const uint8_t*>(row_words) + c);
+    for (int i = 0; i < kBatch; ++i) {
+      const int c = c_lane + 32 * i;
+      if (first + 32 * i >= cpr) break;          // whole warps: at b = 4 the lanes look centroids up for each other
+      uint32_t v = t[i];
+      if constexpr (TUNED && BITS == 2) {
+        // field 4p + c' at bits 2p + 8c'; chunk q of a word holds p = 2q, 2q+1: shift them down to p = 0, 1
+        const uint32_t u = t[i] >> (4 * (c % CPW));
+        v = 0;
+#pragma unroll
+        for (int f = 0; f < 8; ++f) v |= ((u >> field_pos<2>(f, true)) & 3u) << (2 * f);
+      } else if constexpr (TUNED && BITS == 1) {
+        // field 2c' at bit 15 - c', field 2c'+1 at bit 31 - c'; chunk q holds c' = 4q .. 4q+3
+        const uint32_t u = t[i] << (4 * (c % CPW));
+        v = 0;
+#pragma unroll
+        for (int f = 0; f < 8; ++f) v |= ((u >> field_pos<1>(f, true)) & 1u) << f;
       }
       const uint4 w8 = decode8<BITS>(v, c0, c1, row_cb);
-      if (live) stg_stream_u4(out + c, w8);
+      if (c < cpr) stg_stream_u4(out + c, w8);
     }
-  }
+  });
 }
 
 // Table (bit-plane) layout: a thread gathers the plane bytes of one group of 8 weights, interleaves them into
 // LSB-first index fields and stores the 8 decoded weights as one 16-byte piece.
 template <int BITS>
-__global__ void __launch_bounds__(256) dequant_table_kernel(const uint32_t* __restrict__ packed,
-                                                            const uint16_t* __restrict__ cb, uint16_t* __restrict__ W,
-                                                            int64_t N, int64_t K) {
+__global__ void __launch_bounds__(kWarps * 32) dequant_table_kernel(const uint32_t* __restrict__ packed,
+                                                                    const uint16_t* __restrict__ cb,
+                                                                    uint16_t* __restrict__ W, int64_t N, int64_t K,
+                                                                    int shares) {
   constexpr int Q = 1 << BITS;
   const uint8_t* bytes = reinterpret_cast<const uint8_t*>(packed);
   const int gpr = (int)(K >> 3);
   const int64_t chunks = table_chunks(K);
-  for (int64_t n = blockIdx.x; n < N; n += gridDim.x) {
+  for_each_share(N, shares, [&](int64_t n, int first) {
     const uint16_t* row_cb = cb + n * Q;
     uint32_t c0, c1;
     load_codebook<BITS>(row_cb, c0, c1);
-    uint4* out = reinterpret_cast<uint4*>(W + n * K);
-    for (int g = threadIdx.x; g < gpr; g += 256) {
-      uint32_t v = __ldg(bytes + table_byte_offset(n, g, 0, chunks, BITS));
+    uint4* const out = reinterpret_cast<uint4*>(W + n * K);
+    const int g_lane = first + (threadIdx.x & 31);
+    uint32_t plane[kBatch][BITS];
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i)
+#pragma unroll
+      for (int p = 0; p < BITS; ++p)
+        plane[i][p] = g_lane + 32 * i < gpr ? __ldg(bytes + table_byte_offset(n, g_lane + 32 * i, p, chunks, BITS)) : 0;
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int g = g_lane + 32 * i;
+      if (g >= gpr) break;
+      uint32_t v = plane[i][0];
       if constexpr (BITS == 2) {
-        const uint32_t hi = __ldg(bytes + table_byte_offset(n, g, 1, chunks, BITS));
         uint32_t z = 0;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) z |= (((v >> t) & 1u) | (((hi >> t) & 1u) << 1)) << (2 * t);
+        for (int t = 0; t < 8; ++t) z |= (((plane[i][0] >> t) & 1u) | (((plane[i][1] >> t) & 1u) << 1)) << (2 * t);
         v = z;
       }
       stg_stream_u4(out + g, decode8<BITS>(v, c0, c1, row_cb));
     }
-  }
+  });
 }
 
 }  // namespace
 
 cudaError_t launch_dequant(const uint32_t* packed, const uint16_t* cb, uint16_t* W, int64_t N, int64_t K, int bits,
                            int layout, cudaStream_t s) {
-  const DeviceInfo* di = device_info();
-  if (!di) return cudaErrorInvalidDevice;
   const bool tuned = layout != KMQ_LAYOUT_CANONICAL;
-  int64_t blocks = N;
-  const int64_t cap = (int64_t)di->sm_count * 8;   // 8 resident CTAs of 256 threads per SM
-  if (blocks > cap) blocks = cap;
+  const int shares = row_shares(K);
+  const unsigned grid = share_grid(N, K);
+  constexpr int kThreads = kWarps * 32;
   if (layout == KMQ_LAYOUT_TABLE && bits != 4) {
-    if (bits == 1) dequant_table_kernel<1><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-    else dequant_table_kernel<2><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
+    if (bits == 1) dequant_table_kernel<1><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+    else dequant_table_kernel<2><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
     return cudaGetLastError();
   }
-  if (bits == 1 && tuned) dequant_rows_kernel<1, true><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-  else if (bits == 1) dequant_rows_kernel<1, false><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-  else if (bits == 2 && tuned) dequant_rows_kernel<2, true><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-  else if (bits == 2) dequant_rows_kernel<2, false><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-  else if (tuned) dequant_rows_kernel<4, true><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
-  else dequant_rows_kernel<4, false><<<(int)blocks, 256, 0, s>>>(packed, cb, W, N, K);
+  if (bits == 1 && tuned) dequant_rows_kernel<1, true><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+  else if (bits == 1) dequant_rows_kernel<1, false><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+  else if (bits == 2 && tuned) dequant_rows_kernel<2, true><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+  else if (bits == 2) dequant_rows_kernel<2, false><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+  else if (tuned) dequant_rows_kernel<4, true><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
+  else dequant_rows_kernel<4, false><<<grid, kThreads, 0, s>>>(packed, cb, W, N, K, shares);
   return cudaGetLastError();
 }
 
