@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("octaves", (3, 60))
-@pytest.mark.parametrize("members", (1, 31, 32, 33, 64, 200))
+@pytest.mark.parametrize("members", (1, 2, 31, 32, 33, 63, 64, 65, 200))
 def test_members_next_to_zero(members, octaves):
     """`members` values of each sign far below the rest, so that a boundary of the symmetric row lies among them."""
     rng = np.random.default_rng(members + octaves)
