@@ -45,11 +45,11 @@ struct TGeo {
   static constexpr int kStages = 2;                       // steps in flight per warp (deeper rings measured slower)
 };
 
-template <int BITS, int MMAX>
+template <int BITS, int MMAX, int W = kWarps>   // W warps
 struct TSmem {
   using G = TGeo<BITS>;
-  static constexpr int kXs = kWarps * MMAX * G::kRowStride;
-  static constexpr int kRed = kWarps * 32 * 16;
+  static constexpr int kXs = W * MMAX * G::kRowStride;
+  static constexpr int kRed = W * 32 * 16;
   static constexpr int kTotal = G::kTableBytes + kXs + kRed;
 };
 
@@ -61,16 +61,16 @@ __device__ __forceinline__ int piece_offset(int w) {
   return (w / kPiecesPerChunk) * G::kChunkStride + (w % kPiecesPerChunk) * 16;
 }
 
-// Steps [sa, sb) of tile `tile_id`, all 8 warps of the CTA: on return thread i < 128 holds in `v` the sum over those
+// Steps [sa, sb) of tile `tile_id`, all W warps of the CTA: on return thread i < 128 holds in `v` the sum over those
 // steps for output row i % 16 and batch row i / 16.  May be called several times by one CTA; shared memory is reused
 // from call to call.
-template <int BITS, int MMAX>
+template <int BITS, int MMAX, int W = kWarps>
 __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed, const uint16_t* __restrict__ cb,
                                              const uint16_t* x, int64_t N, int64_t K, int M,
                                              int64_t tile_id, int sa, int sb, bool wait_for_x, bool early_trigger,
                                              float& v) {
   using G = TGeo<BITS>;
-  using SM = TSmem<BITS, MMAX>;
+  using SM = TSmem<BITS, MMAX, W>;
   constexpr int Q = G::kMmaPerWord;
   constexpr int STAGES = G::kStages;
   // 16-byte pieces of x per lane and step, and whether they ride in the register ring with the weights
@@ -116,7 +116,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   uint4 qa[STAGES], qb[STAGES], qx[XS][NP];
 #pragma unroll
   for (int d = 0; d < STAGES; ++d) {
-    const int s = sa + warp + d * kWarps;
+    const int s = sa + warp + d * W;
     qa[d] = qb[d] = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int i = 0; i < NP; ++i) qx[kPrefetchX ? d : 0][i] = make_uint4(0, 0, 0, 0);
@@ -142,7 +142,8 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
     // A thread owns one row and one low index: it fetches the row's 16 centroids once (32 bytes) and writes the
     // 16 entries e = low + 16 * high with no further loads.
     const int r8 = threadIdx.x & 7, half = (threadIdx.x >> 3) & 1, low = (threadIdx.x >> 4) & 15;
-    constexpr int kParts = kThreads / 256;   // threads beyond the first 256 take a share of the high indices
+    static_assert(BITS != 4 || W * 32 >= 256, "the tables take 256 threads");
+    constexpr int kParts = W * 32 / 256;   // threads beyond the first 256 take a share of the high indices
     const int part = threadIdx.x >> 8;
     const uint16_t* crow = cb + min(row0 + r8 + 8 * half, N - 1) * 16;
     const uint4 ca = __ldg(reinterpret_cast<const uint4*>(crow)), cc = __ldg(reinterpret_cast<const uint4*>(crow) + 1);
@@ -166,7 +167,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   if (wait_for_x) {
     // a hint only (it binds no value): the first few CTAs pull the activations towards L2 while waiting
     if (blockIdx.x < 4) {
-      for (int64_t o = ((int64_t)blockIdx.x * kThreads + threadIdx.x) * 64; o < (int64_t)M * K; o += 4 * kThreads * 64)
+      for (int64_t o = ((int64_t)blockIdx.x * (W * 32) + threadIdx.x) * 64; o < (int64_t)M * K; o += 4 * (W * 32) * 64)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(x + o));
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -177,7 +178,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   if constexpr (kPrefetchX) {
 #pragma unroll
     for (int d = 0; d < STAGES; ++d) {
-      const int s = sa + warp + d * kWarps;
+      const int s = sa + warp + d * W;
       if (s < sb) load_x(s, qx[d]);
     }
   }
@@ -188,10 +189,10 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
   // g >= M re-read the last real row and their columns are never stored.
   const unsigned char* const xb = xs_warp + min(g, M - 1) * G::kRowStride + t * G::kChunkStride;
 
-  for (int s0 = sa + warp; s0 < sb; s0 += STAGES * kWarps) {
+  for (int s0 = sa + warp; s0 < sb; s0 += STAGES * W) {
 #pragma unroll
     for (int d = 0; d < STAGES; ++d) {
-      const int s = s0 + d * kWarps;
+      const int s = s0 + d * W;
       if (s < sb) {   // warp-uniform
         // stage the activations under this step (zeros past K)
         if constexpr (!kPrefetchX) load_x(s, qx[0]);
@@ -239,7 +240,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
           }
         }
         // refill this stage for the step kStages rounds ahead
-        const int s2 = s + STAGES * kWarps;
+        const int s2 = s + STAGES * W;
         if (s2 < sb) {
           qa[d] = ldg_stream_u4(tile + (int64_t)s2 * 64);
           qb[d] = ldg_stream_u4(tile + (int64_t)s2 * 64 + 32);
@@ -257,7 +258,7 @@ __device__ __forceinline__ void tile_segment(const uint32_t* __restrict__ packed
     const int r = threadIdx.x & 15, m = threadIdx.x >> 4;   // consecutive threads -> consecutive output rows
     const int src_lane = (r & 7) * 4 + (m >> 1), src_reg = (r >> 3) * 2 + (m & 1);
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) v += red[(w * 32 + src_lane) * 4 + src_reg];
+    for (int w = 0; w < W; ++w) v += red[(w * 32 + src_lane) * 4 + src_reg];
   }
 }
 
@@ -317,6 +318,19 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPerSm) linear_tiled_kernel(c
   // weights are under way while this one stores and drains.
   asm volatile("griddepcontrol.launch_dependents;");
   store_output(v, y, N, M, row0);
+}
+
+// The same for short rows, with as many warps as they have steps, so that none is idle, and more CTAs on an SM.
+template <int BITS, int MMAX, int W>
+__global__ void __launch_bounds__(W * 32, 24 / W) linear_tiled_short_kernel(const uint32_t* __restrict__ packed,
+                                                                            const uint16_t* __restrict__ cb,
+                                                                            const uint16_t* x, uint16_t* __restrict__ y,
+                                                                            int64_t N, int64_t K, int M) {
+  const int steps = (int)((uint32_t)(K + TGeo<BITS>::kStepK - 1) / TGeo<BITS>::kStepK);
+  float v;
+  tile_segment<BITS, MMAX, W>(packed, cb, x, N, K, M, blockIdx.x, 0, steps, true, false, v);
+  asm volatile("griddepcontrol.launch_dependents;");
+  store_output(v, y, N, M, (int64_t)blockIdx.x * kRows);
 }
 
 // ---------------------------------------------------------------------------
@@ -422,22 +436,34 @@ int cluster_size(int bits, int64_t tiles, int64_t steps, const DeviceInfo* di, i
   return best;
 }
 
-// CTAs of linear_cluster_kernel<BITS, MMAX> that fit one SM, asked from the runtime once per device and instantiation.
-template <int BITS, int MMAX>
-int cluster_ctas_per_sm() {
+// CTAs of linear_cluster_kernel<BITS, MMAX> (CLUSTER) or linear_tiled_kernel<BITS, MMAX> that fit one SM, asked from the runtime
+// once per device and instantiation.
+template <int BITS, int MMAX, bool CLUSTER>
+int ctas_per_sm() {
   static std::atomic<int> cached[64];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int n = cached[dev].load(std::memory_order_relaxed);
   if (n == 0) {
     constexpr int smem = TSmem<BITS, MMAX>::kTotal;
-    if (cudaFuncSetAttribute(linear_cluster_kernel<BITS, MMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, linear_cluster_kernel<BITS, MMAX>, kThreads, smem) != cudaSuccess)
+    const void* const kernel = CLUSTER ? reinterpret_cast<const void*>(linear_cluster_kernel<BITS, MMAX>)
+                                       : reinterpret_cast<const void*>(linear_tiled_kernel<BITS, MMAX>);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, smem) != cudaSuccess)
       return 0;
     cached[dev].store(n, std::memory_order_relaxed);
   }
   return n;
+}
+
+template <int BITS, int MMAX, int W>
+cudaError_t launch_short(cudaLaunchConfig_t cfg, const uint32_t* packed, const uint16_t* cb, const uint16_t* x, uint16_t* y,
+                         int64_t N, int64_t K, int M) {
+  constexpr int smem = TSmem<BITS, MMAX, W>::kTotal;
+  static_assert(smem <= 48 * 1024, "no need to ask for more");
+  cfg.blockDim = dim3(W * 32);
+  cfg.dynamicSmemBytes = smem;
+  return cudaLaunchKernelEx(&cfg, linear_tiled_short_kernel<BITS, MMAX, W>, packed, cb, x, y, N, K, M);
 }
 
 template <int BITS, int MMAX>
@@ -465,7 +491,7 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   cfg.numAttrs = 1;
   const DeviceInfo* di = device_info();
   const int64_t steps = tuned_row_steps(K, BITS);
-  if (const int C = cluster_size(BITS, (N + kRows - 1) / kRows, steps, di, cluster_ctas_per_sm<BITS, MMAX>()); C > 1) {
+  if (const int C = cluster_size(BITS, (N + kRows - 1) / kRows, steps, di, ctas_per_sm<BITS, MMAX, true>()); C > 1) {
     cfg.gridDim.x *= C;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)C;
@@ -474,6 +500,22 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
     cfg.numAttrs = 2;
     const int early = early_trigger(BITS, (N + kRows - 1) / kRows * C, steps / C, di->sm_count) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, linear_cluster_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M, early, C);
+  }
+  // Rows of up to four steps (b = 1: six) leave warps of eight idle.  Where the tiles do not all find room at once, a CTA of as many
+  // warps as steps makes room for half as many again; where they do, warps that have nothing to decode do no harm (b = 2, up to
+  // 10 % slower with four).  us per call, eight warps / as many as steps: b = 2 16384 x 512, M = 2 4.93 / 2.82, 9500 x 1024, M = 1
+  // 3.25 / 2.58, 8192 x 256, M = 3 3.15 / 1.99, but 8192 x 1024, M = 1 (512 tiles, four CTAs an SM) 2.38 / 2.59; b = 1 16384 x 1024
+  // 5.92 / 3.48, 9500 x 3072 5.53 / 5.12.  Six warps at b = 1, M = 1 also with room for all: 3072 x 3072 3.20 / 2.81, a decode step
+  // of 1536 / 4096 257.9 / 231.2; with more rows, between calls of the multi-tile kernel, they gain nothing (3072 / 8192, M = 2
+  // 271.4 / 276.5).
+  if constexpr (BITS != 4 && MMAX <= 4) {   // (more rows of many tiles are the multi-tile kernel's)
+    const int per_sm = ctas_per_sm<BITS, MMAX, false>();
+    const bool crowded = di && per_sm > 0 && (N + kRows - 1) / kRows > (int64_t)per_sm * di->sm_count;
+    if (steps <= 4 && crowded) return launch_short<BITS, MMAX, 4>(cfg, packed, cb, x, y, N, K, M);
+    if constexpr (BITS == 1) {
+      if (steps == 6 ? MMAX == 1 || crowded : steps == 5 && crowded)
+        return launch_short<BITS, MMAX, 6>(cfg, packed, cb, x, y, N, K, M);
+    }
   }
   const int early = di && early_trigger(BITS, (N + kRows - 1) / kRows, steps, di->sm_count) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, linear_tiled_kernel<BITS, MMAX>, packed, cb, x, y, N, K, M, early);
