@@ -227,8 +227,8 @@ size_t kmq_static_scratch_capacity(void);
  * the layer is compute bound).  A CTA covers 128 output rows and up to 128
  * batch rows; beyond that, where it pays, pairs of CTAs share tiles of 256 rows
  * by up to 256 batch rows.  kmq_linear itself selects this kernel for M > 32,
- * and from M = 9 on unless rows are short and few
- * (kmq_linear_variant() then starts with "tcgen05"); this entry point forces
+ * from M = 9 on unless rows are short and few, and at b = 4 and 2 for fewer
+ * batch rows where rows are long and many (kmq_linear_variant() then starts with "tcgen05"); this entry point forces
  * it for any shape.
  * packed and codebooks may be read before earlier work on `stream` has
  * finished, as by kmq_linear, with the same condition on the kernel that
