@@ -5,6 +5,7 @@
 // grid that stays resident, with equal shares for all, ends with the slowest (470 MB of plain stores: 76.6 us from 1184 CTAs
 // in a loop, 64 to 68 us from 9472 and more).  8192 x 28672, b = 4 106.0 -> 92.4 us.
 #include "kmq_common.cuh"
+#include "kmq_mma_common.cuh"
 #include "kmq_table_layout.cuh"
 
 namespace kmq {
@@ -43,6 +44,31 @@ __device__ __forceinline__ uint4 decode8(uint32_t v, uint32_t c0, uint32_t c1, c
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// 8 weights of the tuned layout (b = 1, 2), whose fields lie where few instructions take several: one shift and the decoders of
+// the tensor-core kernels.  Cutting the fields out one by one and putting them back in order for decode8 took more integer
+// instructions than the stores left time for: 8192 x 28672, b = 1 100.5 us, so 76.2; b = 2 96.5, so 82.8.
+template <int BITS>
+struct TunedDecoder {};
+template <>
+struct TunedDecoder<1> : Dec1 {
+  // fields 2c', 2c'+1 at bits 15 - c', 31 - c'; chunk q holds c' = 4q .. 4q+3
+  __device__ __forceinline__ uint4 chunk(uint32_t t, int q) const {
+    const uint32_t u = t << (4 * q);
+    return make_uint4(select(u), select(u << 1), select(u << 2), select(u << 3));
+  }
+};
+template <>
+struct TunedDecoder<2> : Dec2 {
+  // field 4p + c' at bits 2p + 8c'; chunk q holds p = 2q, 2q+1
+  __device__ __forceinline__ uint4 chunk(uint32_t t, int q) const {
+    const uint32_t u = t >> (4 * q);
+    uint4 o;
+    pair(u, 0, o.x, o.y);
+    pair(u, 1, o.z, o.w);
+    return o;
+  }
+};
+
 template <int BITS>
 __device__ __forceinline__ void load_codebook(const uint16_t* __restrict__ row_cb, uint32_t& c0, uint32_t& c1) {
   c0 = c1 = 0;
@@ -74,8 +100,7 @@ __device__ __forceinline__ void for_each_share(int64_t N, int shares, F f) {
   }
 }
 
-// In the tuned layout the row's words come in 64-byte runs, one per 1 KB step of its tile, and the 8 fields of a chunk are
-// cut out of the word after one shift.
+// In the tuned layout the row's words come in 64-byte runs, one per 1 KB step of its tile.
 template <int BITS, bool TUNED>
 __global__ void __launch_bounds__(kWarps * 32) dequant_rows_kernel(const uint32_t* __restrict__ packed,
                                                                    const uint16_t* __restrict__ cb,
@@ -90,8 +115,11 @@ __global__ void __launch_bounds__(kWarps * 32) dequant_rows_kernel(const uint32_
     const uint32_t* row_words =
         TUNED ? packed + ((n >> 4) * steps * kTileRows + (n & 15)) * 16 : packed + n * wpr;
     const uint16_t* row_cb = cb + n * Q;
+    constexpr bool kFields = TUNED && BITS != 4;
+    TunedDecoder<kFields ? BITS : 1> dec;
     uint32_t c0, c1;
-    load_codebook<BITS>(row_cb, c0, c1);
+    if constexpr (kFields) dec.init(row_cb);
+    else load_codebook<BITS>(row_cb, c0, c1);
     uint4* const out = reinterpret_cast<uint4*>(W + n * K);
     const int c_lane = first + (threadIdx.x & 31);
     uint32_t t[kBatch];
@@ -109,28 +137,20 @@ __global__ void __launch_bounds__(kWarps * 32) dequant_rows_kernel(const uint32_
     for (int i = 0; i < kBatch; ++i) {
       const int c = c_lane + 32 * i;
       if (first + 32 * i >= cpr) break;          // whole warps: at b = 4 the lanes look centroids up for each other
-      uint32_t v = t[i];
-      if constexpr (TUNED && BITS == 2) {
-        // field 4p + c' at bits 2p + 8c'; chunk q of a word holds p = 2q, 2q+1: shift them down to p = 0, 1
-        const uint32_t u = t[i] >> (4 * (c % CPW));
-        v = 0;
-#pragma unroll
-        for (int f = 0; f < 8; ++f) v |= ((u >> field_pos<2>(f, true)) & 3u) << (2 * f);
-      } else if constexpr (TUNED && BITS == 1) {
-        // field 2c' at bit 15 - c', field 2c'+1 at bit 31 - c'; chunk q holds c' = 4q .. 4q+3
-        const uint32_t u = t[i] << (4 * (c % CPW));
-        v = 0;
-#pragma unroll
-        for (int f = 0; f < 8; ++f) v |= ((u >> field_pos<1>(f, true)) & 1u) << f;
-      }
-      const uint4 w8 = decode8<BITS>(v, c0, c1, row_cb);
+      uint4 w8;
+      if constexpr (kFields) w8 = dec.chunk(t[i], c % CPW);
+      else w8 = decode8<BITS>(t[i], c0, c1, row_cb);
       if (c < cpr) stg_stream_u4(out + c, w8);
     }
   });
 }
 
-// Table (bit-plane) layout: a thread gathers the plane bytes of one group of 8 weights, interleaves them into
-// LSB-first index fields and stores the 8 decoded weights as one 16-byte piece.
+// Four bits -> the lowest bits of four bytes.
+__device__ __forceinline__ uint32_t spread(uint32_t nibble) { return (nibble & 15u) * 0x00204081u; }
+
+// Table (bit-plane) layout: a thread gathers the plane bytes of one group of 8 weights and stores the 8 decoded weights as one
+// 16-byte piece.  b = 2: the planes' bits are spread to the bytes of a word of four indices by multiplies; bit by bit 8192 x 28672
+// took 108 us, so 92.6.
 template <int BITS>
 __global__ void __launch_bounds__(kWarps * 32) dequant_table_kernel(const uint32_t* __restrict__ packed,
                                                                     const uint16_t* __restrict__ cb,
@@ -142,8 +162,10 @@ __global__ void __launch_bounds__(kWarps * 32) dequant_table_kernel(const uint32
   const int64_t chunks = table_chunks(K);
   for_each_share(N, shares, [&](int64_t n, int first) {
     const uint16_t* row_cb = cb + n * Q;
+    Dec2 dec;
     uint32_t c0, c1;
-    load_codebook<BITS>(row_cb, c0, c1);
+    if constexpr (BITS == 2) dec.init(row_cb);
+    else load_codebook<BITS>(row_cb, c0, c1);
     uint4* const out = reinterpret_cast<uint4*>(W + n * K);
     const int g_lane = first + (threadIdx.x & 31);
     uint32_t plane[kBatch][BITS];
@@ -156,14 +178,14 @@ __global__ void __launch_bounds__(kWarps * 32) dequant_table_kernel(const uint32
     for (int i = 0; i < kBatch; ++i) {
       const int g = g_lane + 32 * i;
       if (g >= gpr) break;
-      uint32_t v = plane[i][0];
       if constexpr (BITS == 2) {
-        uint32_t z = 0;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) z |= (((plane[i][0] >> t) & 1u) | (((plane[i][1] >> t) & 1u) << 1)) << (2 * t);
-        v = z;
+        uint4 o;
+        dec.pair((spread(plane[i][0]) & 0x01010101u) | (spread(plane[i][1]) << 1 & 0x02020202u), 0, o.x, o.y);
+        dec.pair((spread(plane[i][0] >> 4) & 0x01010101u) | (spread(plane[i][1] >> 4) << 1 & 0x02020202u), 0, o.z, o.w);
+        stg_stream_u4(out + g, o);
+      } else {
+        stg_stream_u4(out + g, decode8<BITS>(plane[i][0], c0, c1, row_cb));
       }
-      stg_stream_u4(out + g, decode8<BITS>(v, c0, c1, row_cb));
     }
   });
 }
