@@ -227,9 +227,11 @@ size_t kmq_static_scratch_capacity(void);
  * the layer is compute bound).  A CTA covers 128 output rows and up to 128
  * batch rows; beyond that, where it pays, pairs of CTAs share tiles of 256 rows
  * by up to 256 batch rows.  kmq_linear itself selects this kernel for M > 32,
- * from M = 9 on unless rows are short and few, and at b = 4 and 2 for fewer
- * batch rows where rows are long and many (kmq_linear_variant() then starts with "tcgen05"); this entry point forces
- * it for any shape.
+ * from M = 9 on unless rows are short and few, and for fewer batch rows (b = 4,
+ * from M = 6 on b = 2) where it is the faster one: rows long for their number,
+ * from 2048 weights where blocks of 128 rows take two thirds of the SMs to 8192
+ * with 8 blocks; kmq_linear_variant() then starts with "tcgen05".  This entry
+ * point forces it for any shape.
  * packed and codebooks may be read before earlier work on `stream` has
  * finished, as by kmq_linear, with the same condition on the kernel that
  * writes them.

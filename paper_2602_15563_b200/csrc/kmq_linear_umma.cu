@@ -594,17 +594,18 @@ bool linear_umma_few_rows(int64_t N, int64_t K, int bits, int64_t M) {
   const DeviceInfo* di = device_info();
   if (!di || M > 8 || !encode_tiled()) return false;
   const int64_t sms = di->sm_count, blocks = (N + kBM - 1) / kBM, waves = (blocks + sms - 1) / sms;
-  if (blocks < 8) return false;                            // the GEMV kernel's clusters fill the machine with them
+  const int64_t part = 1000 * blocks / sms;                // thousandths of the SMs that have a block
+  if (part < 50) return false;                             // the GEMV kernel's clusters fill the machine with so few
   const int64_t filled = 100 * blocks / (waves * sms);     // % of the machine, one CTA a block
   const bool half = 2 * blocks <= sms;                     // room for two CTAs a block
   if (bits == 4 && M > 2) {
     if (!half) return filled >= 64 ? K >= 2048 : filled >= 55 && K >= 4096;
-    if (blocks >= 53) return K >= (M <= 5 ? 6144 : 4096);
-    if (blocks >= 40) return K >= 3072;
+    if (part >= 355) return K >= (M <= 5 ? 6144 : 4096);
+    if (part >= 267) return K >= 3072;
     return K >= (M <= 5 ? 8192 : 6144);
   }
   if (bits == 1 || N * K < (int64_t(1) << 26)) return false;
-  if (bits == 4) return !half ? filled >= 64 : blocks >= 56 || blocks <= 40;
+  if (bits == 4) return !half ? filled >= 64 : part >= 375 || part <= 272;   // between: a cluster of two leaves too many SMs empty
   return M >= 6 && filled >= 75;
 }
 
