@@ -2,10 +2,12 @@
 results; row lengths that leave CTAs of a cluster one stage or none at the end."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import kmq_oracle as orc
 from paper_2602_15563_b200 import kmq
 from tests import gpu_util as gu
+from tests.test_gpu_sum_error import layer
 from tests.test_gpu_tcgen05 import random_layer
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +38,17 @@ def test_few_rows_on_either_side_of_a_line(bits, N, K, M, tcgen05):
     y_ref, s = orc.linear_f64(orc.pack_canonical(idx[rows], bits), cb[rows], x, K, bits)
     assert orc.check_linear(y[:, rows], y_ref, s) <= 1.0
     assert kmq.kmq_device_error_flags() == 0
+
+
+@pytest.mark.parametrize("bits,N,K,M", [(4, 8192, 8192, 1), (4, 12033, 5640, 2), (4, 4312, 9216, 3), (4, 8259, 13696, 3),
+                                        (4, 900, 28672, 8), (4, 5120, 28672, 1), (4, 4378, 21344, 5), (4, 12033, 2048, 8),
+                                        (2, 16384, 8192, 8)])
+def test_share_of_results_that_are_not_the_rounded_exact_ones(bits, N, K, M):
+    """The bound of 9 to 16 batch rows, which run in the same form (8 accumulators): see tests/test_gpu_sum_error.py."""
+    packed, cb, x, exact = layer(bits, N, K, M)
+    assert kmq.kmq_linear_variant(N, K, bits, M, TUNED).startswith("tcgen05")
+    y = torch.zeros(M, N, dtype=torch.bfloat16, device="cuda")
+    kmq.kmq_linear(packed, cb, x, y, N, K, bits, M, None, 0, layout=TUNED)
+    off = int((y != exact.float().to(torch.bfloat16)).sum())
+    expected = (1.5 * 7.6e-6 * (K / 16) / 8 + 1e-4) * M * N
+    assert off <= expected + 4 * expected ** 0.5     # few results: four standard deviations of their number
