@@ -505,9 +505,9 @@ cudaError_t launch_one(const uint32_t* packed, const uint16_t* cb, const uint16_
   // warps as steps makes room for half as many again; where they do, warps that have nothing to decode do no harm (b = 2, up to
   // 10 % slower with four).  us per call, eight warps / as many as steps: b = 2 16384 x 512, M = 2 4.93 / 2.82, 9500 x 1024, M = 1
   // 3.25 / 2.58, 8192 x 256, M = 3 3.15 / 1.99, but 8192 x 1024, M = 1 (512 tiles, four CTAs an SM) 2.38 / 2.59; b = 1 16384 x 1024
-  // 5.92 / 3.48, 9500 x 3072 5.53 / 5.12.  Six warps at b = 1, M = 1 also with room for all: 3072 x 3072 3.20 / 2.81, a decode step
-  // of 1536 / 4096 257.9 / 231.2; with more rows, between calls of the multi-tile kernel, they gain nothing (3072 / 8192, M = 2
-  // 271.4 / 276.5).
+  // 5.92 / 3.48, 9500 x 3072 5.53 / 5.12.  Six warps at b = 1, M = 1 also with room for all: over 2592, 2880 and 3072 weights and 256 to 12288 rows 11 to 18 %
+  // faster from 2560 to 4736 rows and from 8192 on (3072 x 3072 3.10 / 2.75), elsewhere the same (0.4 %); a decode step of 3072 / 8192,
+  // 16 layers, 332 / 302.  With more rows, between calls of the multi-tile kernel, they gain nothing (that step, M = 2, 361 / 361).
   if constexpr (BITS != 4 && MMAX <= 4) {   // (more rows of many tiles are the multi-tile kernel's)
     const int per_sm = ctas_per_sm<BITS, MMAX, false>();
     const bool crowded = di && per_sm > 0 && (N + kRows - 1) / kRows > (int64_t)per_sm * di->sm_count;

@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_umma_kernel(const uint32_t
         }
         // The words of the stage before are loaded anew only now that this stage's have arrived: a wait for registers of a load
         // is a wait for later loads too, where they share one of a warp's few counters, and behind the stage's decode each
-        // round ended with the latency of the load just issued.  us, before / now: 8192 x 28672, M = 16, b = 4 29.4 / 28.1,
-        // b = 2 31.9 / 30.2; at b = 1, with eight loads of one word each in flight, 28.1 / 28.4.
+        // round ended with the latency of the load just issued.  us in a graph, before / now: 8192 x 28672, M = 16, b = 4 29.6 / 28.3,
+        // b = 2 32.2 / 30.5; at b = 1, with eight loads of one word each in flight, it gained nothing (28.4 as before).
         if constexpr (BITS >= 2) {
           arrived<NW>(words[p]);
           if (i != group && i + (kAhead - 1) * kGroups < total)
